@@ -49,11 +49,19 @@ int sm_count_of(int device) {
     return c;
 }
 
-// Chunk length k: one reach thread per chunk, about 2 resident warps per
-// scheduler, chunks long enough that speculative runs meet early in them.
-uint32_t choose_chunk(uint64_t n, int sms, const re_parse_opts *opts) {
+// The lane walk (RE_PARSE_REACH shape 1) is the built-in choice for automata of
+// at most 256 states whose two-byte tables do not fit shared memory.
+bool walks(const re_handle *h);
+uint32_t table_mode(const DevTables &t);
+
+// Chunk length k.  Lane walk: a lane per chunk, as many chunks as the device
+// walks at once in a direction.  Otherwise one reach thread per chunk, about 2
+// resident warps per scheduler, chunks long enough that speculative runs meet
+// early in them.
+uint32_t choose_chunk(const re_handle *h, uint64_t n, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
-    const uint64_t target = (uint64_t)sms * 384;
+    const bool rec = opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY);
+    const uint64_t target = walks(h) && table_mode(h->dev) == TM_SMEM ? walk_lanes(h->dev, rec, sms) : (uint64_t)sms * 384;
     uint64_t k = (n + target - 1) / target;
     k = (k + kSub - 1) / kSub * kSub;
     return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(k, 256), 1u << 20);
@@ -84,10 +92,9 @@ uint32_t tuned_shape(re_handle *h, uint64_t n, const re_parse_opts *opts) {
 
 // Reach shapes this handle can run (bit v: shape v of RE_PARSE_REACH).
 uint32_t shapes_of(const re_handle *h) {
-    uint32_t m = (1u << 2) | (1u << 3) | (1u << 4);
-    if (!h->host.fbyte.empty() && !h->host.bbyte.empty()) m |= 1u << 1;
-    return m;
+    return (1u << 2) | (1u << 3) | (1u << 4) | (walks(h) ? 1u << 1 : 0u);
 }
+bool walks(const re_handle *h) { return !h->host.fc8.empty(); }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -106,16 +113,18 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 // Text viewed as rows of full chunks (k bytes), one box = 32 chunks x 64
-// bytes, SWIZZLE_64B to match the reach kernel's tile reads.
-bool text_tensor_map(CUtensorMap &map, const uint8_t *d_text, uint32_t k, uint64_t rows) {
+// bytes, SWIZZLE_64B to match the reach kernel's tile reads; the lane walk's
+// boxes are 32 bytes wide (SWIZZLE_32B).
+bool text_tensor_map(CUtensorMap &map, const uint8_t *d_text, uint32_t k, uint64_t rows, uint32_t width = 64) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
     if (!fn || rows < 32 || rows > 0x7FFFFFFFull || (k % 64) != 0) return false;   // int32 row coordinates
     const cuuint64_t dims[2] = {k, rows};
     const cuuint64_t strides[1] = {k};
-    const cuuint32_t box[2] = {64u, 32u};
+    const cuuint32_t box[2] = {width, 32u};
     const cuuint32_t estr[2] = {1u, 1u};
     const CUresult r = fn(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(d_text), dims, strides, box,
-                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          width == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -316,11 +325,13 @@ re_status re_compile(const char *pattern, size_t len, const re_compile_opts *opt
     const size_t i_bSM = add(C.bSlotMask.data(), C.bSlotMask.size() * 8);
     const size_t i_bSC = add(C.bSlotCount.data(), C.bSlotCount.size() * 4);
     const size_t i_pt = add(C.pt.data(), C.pt.size() * 4);
+    const size_t i_ptc = add(C.ptc.data(), C.ptc.size());
     const size_t i_f2 = add(C.f2.data(), C.f2.size() * 4), i_b2 = add(C.b2.data(), C.b2.size() * 4);
     const size_t i_fs = add(C.folseg.data(), C.folseg.size() * 8), i_dc = add(C.dict.data(), C.dict.size() * 8);
     const size_t i_fso = add(C.fSlotOf.data(), C.fSlotOf.size());
     const size_t i_bso = add(C.bSlotOf.data(), C.bSlotOf.size());
     const size_t i_fby = add(C.fbyte.data(), C.fbyte.size()), i_bby = add(C.bbyte.data(), C.bbyte.size());
+    const size_t i_fc8 = add(C.fc8.data(), C.fc8.size()), i_bc8 = add(C.bc8.data(), C.bc8.size());
     const size_t i_hr = add(C.hirep.data(), C.hirep.size());
     DevTables &t = h->dev;
     t.fHashMask = C.fHashMask; t.bHashMask = C.bHashMask;
@@ -348,6 +359,7 @@ re_status re_compile(const char *pattern, size_t len, const re_compile_opts *opt
     t.bSlotStart = (const uint32_t *)(b + pc[i_bSS].off); t.bSlotMask = (const uint64_t *)(b + pc[i_bSM].off);
     t.bSlotCount = (const uint32_t *)(b + pc[i_bSC].off);
     t.pt = (const uint32_t *)(b + pc[i_pt].off);
+    t.ptc = C.ptc.empty() ? nullptr : b + pc[i_ptc].off;
     t.fSlotOf = C.fSlotOf.empty() ? nullptr : (const uint8_t *)(b + pc[i_fso].off);
     t.bSlotOf = C.bSlotOf.empty() ? nullptr : (const uint8_t *)(b + pc[i_bso].off);
     t.f2 = C.f2.empty() ? nullptr : (const uint32_t *)(b + pc[i_f2].off);
@@ -355,6 +367,8 @@ re_status re_compile(const char *pattern, size_t len, const re_compile_opts *opt
     t.folseg = (const uint64_t *)(b + pc[i_fs].off);
     t.fbyte = C.fbyte.empty() ? nullptr : b + pc[i_fby].off;
     t.bbyte = C.bbyte.empty() ? nullptr : b + pc[i_bby].off;
+    t.fc8 = C.fc8.empty() ? nullptr : b + pc[i_fc8].off;
+    t.bc8 = C.bc8.empty() ? nullptr : b + pc[i_bc8].off;
     t.hirep = C.hirep.empty() ? nullptr : b + pc[i_hr].off;
     t.dict = C.dict.empty() ? nullptr : (const uint64_t *)(b + pc[i_dc].off);
     *out = h;
@@ -417,7 +431,7 @@ re_status re_slpf_layout(const re_handle *h, uint64_t len, re_slpf_kind kind, re
 re_status re_workspace_size(const re_handle *h, uint64_t len, const re_parse_opts *opts, uint64_t *bytes) {
     if (!h || !bytes) { set_error("null argument"); return RE_E_INVALID_ARG; }
     const uint32_t kt = tuned_chunk(const_cast<re_handle *>(h), len, opts);
-    const uint32_t k = kt ? kt : choose_chunk(len, sm_count_of(h->device), opts);
+    const uint32_t k = kt ? kt : choose_chunk(h, len, sm_count_of(h->device), opts);
     if (k % kSub || k == 0) { set_error("chunk_len must be a positive multiple of 64"); return RE_E_INVALID_ARG; }
     *bytes = layout_for(h, len, k, mat_for(h, opts)).total;
     return RE_OK;
@@ -430,7 +444,7 @@ namespace slpf {
 // what re_parse falls back to when the workspace it is given cannot hold the
 // tuned layout.
 re_status workspace_rule_bytes(const re_handle *h, uint64_t len, const re_parse_opts *opts, uint64_t *bytes) {
-    const uint32_t k = choose_chunk(len, sm_count_of(h->device), opts);
+    const uint32_t k = choose_chunk(h, len, sm_count_of(h->device), opts);
     if (k % kSub || k == 0) { set_error("chunk_len must be a positive multiple of 64"); return RE_E_INVALID_ARG; }
     *bytes = layout_for(h, len, k, mat_for(h, opts)).total;
     return RE_OK;
@@ -501,7 +515,7 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     cudaGetDevice(&dev_now);
     if (dev_now != h->device) { set_error("current device differs from the handle's device"); return RE_E_INVALID_ARG; }
     const int sms = sm_count_of(h->device);
-    uint32_t k = choose_chunk(len, sms, opts);
+    uint32_t k = choose_chunk(h, len, sms, opts);
     if (const uint32_t kt = tuned_chunk(h, len, opts)) {      // tuned length, if the workspace holds it
         if (!len || layout_for(h, len, kt, mat_for(h, opts)).total <= workspace_bytes) k = kt;
     }
@@ -557,19 +571,25 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     alignas(64) CUtensorMap text_map;
     std::memset(&text_map, 0, sizeof(text_map));
     p.c_full = (uint32_t)(len / k);
-    p.text_tma = text_tensor_map(text_map, d_text, k, p.c_full) ? 1u : 0u;
-    // Per-position states: the reach writes them, the fix-up fills the heads,
-    // build & merge gathers (when the gather's encoder fits shared memory).
+    // Per-position states: the reach writes them, build & merge gathers (when
+    // the gather's encoder fits shared memory).  The lane walk needs them for
+    // columns; without them shape 2 takes its place.
+    const bool mat_fits = mat_ws && len && mat_gather_smem(p) <= kSmemMergeMax;
+    const bool lane_walk = shape == 1 && (recognize || mat_fits);
+    if (shape == 1 && !lane_walk) p.rvar = shape = 2;
+    p.text_tma = text_tensor_map(text_map, d_text, k, p.c_full, lane_walk ? 32 : 64) ? 1u : 0u;
     alignas(64) StateMaps smaps;
     std::memset(&smaps, 0, sizeof(smaps));
-    if (mat_ws && len && shape_stores_states(h, shape) && mat_gather_smem(p) <= kSmemMergeMax) {
+    if (mat_fits && shape_stores_states(h, shape)) {
         p.mat = 1;
         uint8_t *w = (uint8_t *)d_workspace;
-        const bool maps = p.text_tma && text_tensor_map(smaps.f, w + L.off[24], k, p.c_full) &&
-                          text_tensor_map(smaps.b, w + L.off[25], k, p.c_full);
+        const uint32_t width = lane_walk ? 32u : 64u;
+        const bool maps = p.text_tma && text_tensor_map(smaps.f, w + L.off[24], k, p.c_full, width) &&
+                          text_tensor_map(smaps.b, w + L.off[25], k, p.c_full, width);
         if (!maps) p.text_tma = 0;                            // state rows and text tiles use the same path
         p.state_tma = p.text_tma;
     }
+    p.rall = map_mode ? 1u : 0u;
     auto mark = [&](int j) -> cudaError_t { return ev ? cudaEventRecord(ev[j], s) : cudaSuccess; };
     if (len == 0) {
         CUDA_TRY(mark(0), "event");
@@ -580,10 +600,15 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     }
     carve(p, L, (uint8_t *)d_workspace);
     CUDA_TRY(mark(0), "event");
-    launch_flags_init(p, s);
-    if (!launch_reach(p, text_map, smaps, s, std::max(t.msf, p.recognize ? 1u : t.msb), sms)) {
-        set_error("too many speculative starts");
-        return RE_E_INTERNAL;
+    if (lane_walk) {
+        launch_heads(p, s, sms);
+        launch_walk(p, text_map, smaps, s, sms);
+    } else {
+        launch_flags_init(p, s);
+        if (!launch_reach(p, text_map, smaps, s, std::max(t.msf, p.recognize ? 1u : t.msb), sms)) {
+            set_error("too many speculative starts");
+            return RE_E_INTERNAL;
+        }
     }
     CUDA_TRY(mark(1), "event");
     if (map_mode) {                                           // the slice's maps, no columns
@@ -592,10 +617,11 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
         CUDA_TRY(cudaGetLastError(), "launch");
         return RE_OK;
     }
-    if (!launch_join(p, s, sms)) return cuda_fail(cudaGetLastError(), "join launch");
+    if (!(lane_walk ? launch_join_walk(p, s, sms) : launch_join(p, s, sms)))
+        return cuda_fail(cudaGetLastError(), "join launch");
     CUDA_TRY(mark(2), "event");
     if (!recognize) {
-        launch_fixup(p, s, sms);
+        if (!lane_walk) launch_fixup(p, s, sms);              // the walk has been through the chunk heads
         CUDA_TRY(mark(3), "event");
         launch_merge(p, out_map, s, sms);
     } else {
@@ -615,7 +641,7 @@ extern "C" re_status re_autotune(re_handle *h, const uint8_t *d_text, uint64_t l
     if (opts && opts->chunk_len) { set_error("autotune chooses chunk_len: pass 0"); return RE_E_INVALID_ARG; }
     if (opts && opts->n_events) { set_error("autotune records its own events"); return RE_E_INVALID_ARG; }
     if (opts && (opts->flags & RE_PARSE_REACH_MASK)) { set_error("autotune chooses the reach shape"); return RE_E_INVALID_ARG; }
-    const uint32_t k0 = choose_chunk(len, sm_count_of(h->device), nullptr);
+    const uint32_t k0 = choose_chunk(h, len, sm_count_of(h->device), opts);
     std::vector<uint32_t> cand;
     for (uint32_t num : {2u, 3u, 4u, 5u, 6u, 8u}) {            // k0 * num / 4, multiples of 64, >= 256
         uint64_t k = (uint64_t)k0 * num / 4;
@@ -627,17 +653,12 @@ extern "C" re_status re_autotune(re_handle *h, const uint8_t *d_text, uint64_t l
     std::vector<uint32_t> shapes;                              // every reach shape this automaton can run
     for (uint32_t v = 1; v <= 4; ++v)
         if (shapes_of(h) >> v & 1) shapes.push_back(v);
-    if (!h->host_only && (shapes_of(h) >> 1 & 1)) {
-        // Whole rounds of tiles: with m tiles for every warp of the byte-table
-        // reach, no warp idles while others walk a last tile.
-        Params q{};
-        q.t = h->dev;
-        q.recognize = (opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY)) ? 1u : 0u;
-        q.mat = mat_for(h, opts) ? 1u : 0u;
-        const uint32_t ms = std::max(h->dev.msf, q.recognize ? 1u : h->dev.msb);
-        const uint64_t warps = reach_byte8_warps(q, ms, sm_count_of(h->device));
-        for (uint64_t m = 1; m <= 4 && warps; ++m) {
-            uint64_t k = (len + 32 * warps * m - 1) / (32 * warps * m);
+    if (!h->host_only && walks(h)) {
+        // Whole rounds of tiles: with m tiles for every warp of the lane walk,
+        // no warp idles while others walk a last tile.
+        const uint64_t lanes = walk_lanes(h->dev, opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY), sm_count_of(h->device));
+        for (uint64_t m = 1; m <= 4; ++m) {
+            uint64_t k = (len + lanes * m - 1) / (lanes * m);
             k = (k + kSub - 1) / kSub * kSub;
             if (k < 256 || k > (1u << 20) || std::find(cand.begin(), cand.end(), (uint32_t)k) != cand.end()) continue;
             if (layout_for(h, len, (uint32_t)k, mat_for(h, opts)).total > workspace_bytes) continue;
@@ -890,9 +911,9 @@ namespace {
 // group's total bytes (one reach lane per chunk, about one wave of lanes for
 // the whole group), but short enough that the text spans a warp tile of 32
 // chunks where it can.
-uint32_t batch_chunk(uint64_t len, uint64_t group_bytes, int sms, const re_parse_opts *opts) {
+uint32_t batch_chunk(const re_handle *h, uint64_t len, uint64_t group_bytes, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
-    const uint32_t kg = choose_chunk(group_bytes, sms, nullptr);
+    const uint32_t kg = choose_chunk(h, group_bytes, sms, nullptr);
     uint64_t kt = (len + 31) / 32;
     kt = (kt + kSub - 1) / kSub * kSub;
     return (uint32_t)std::max<uint64_t>(256, std::min<uint64_t>(kg, kt));
@@ -1013,7 +1034,7 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
     // chunk lengths, then members longest chunks first
     for (uint32_t j = 0; j < count; ++j) {
         re_batch::Text &t = b->texts[j];
-        t.k = batch_chunk(t.len, gbytes[t.group], b->sms, opts);
+        t.k = batch_chunk(b->groups[t.group].h, t.len, gbytes[t.group], b->sms, opts);
         if (t.len / t.k >= 0xFFFFFFF0ull) { set_error("text too long for this chunk length"); return RE_E_INVALID_ARG; }
         if (t.len) t.L = layout_for(b->groups[t.group].h, t.len, t.k, b->groups[t.group].mat);
     }

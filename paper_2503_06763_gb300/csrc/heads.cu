@@ -1,0 +1,285 @@
+// Speculative chunk heads (arXiv 2503.06763, Eq. reacher and Sect. 4.3; see
+// walk.cuh).
+//
+// For every chunk and direction the speculative runs are walked from the
+// chunk's edge until the live ones are in one state, checked every kUnit
+// bytes; the state, the unit boundary it holds at and the slots alive there
+// are recorded.  The chunk's slots are those of the class pair around its edge
+// (the start sets after the boundary byte, the last-character filter of Sect.
+// 6).  A chunk whose runs never meet (kind 1) is walked to its end here and
+// leaves every slot's end state to the join.
+//
+// A block takes up to kHeadChunks chunks of one direction.  Their first bytes
+// come into shared memory together (the walk itself then waits for no text:
+// on most chunks it ends within them).  A chunk with more slots than a lane
+// holds in registers (kRuns) is first taken by a whole warp, a lane per slot,
+// until few enough states are left: on log text 8 slots on average (at most
+// 23) are 2.4 states after 4 bytes and 1.6 after 32, so that is a few bytes.
+// Then a lane walks the chunk's runs.  The loops are rolled, a word of text a
+// turn: unrolled over a unit the kernel spent a third of its time fetching
+// instructions.
+#include <algorithm>
+#include <type_traits>
+
+#include "walk.cuh"
+
+namespace slpf {
+namespace {
+
+constexpr uint32_t kHeadThreads = 256;
+constexpr uint32_t kHeadChunks = 64;        // chunks a block takes at once, at most
+constexpr uint32_t kHeadWindow = 144;       // bytes of a chunk staged, from its edge (a multiple of 16)
+constexpr uint32_t kHeadStride = 148;       // their stride: an odd number of words, so lanes hit different banks
+constexpr int kRuns = 4;
+
+// Drop dead runs and merge runs in equal states (their slot sets are joined);
+// unused runs hold the empty state.
+__device__ __forceinline__ void merge_runs(uint32_t (&s)[kRuns], uint32_t (&k)[kRuns], uint32_t &cnt) {
+    uint32_t ns[kRuns] = {}, nk[kRuns] = {};
+    cnt = 0;
+#pragma unroll
+    for (int j = 0; j < kRuns; ++j) {
+        if (!s[j]) continue;
+        bool merged = false;
+#pragma unroll
+        for (int q = 0; q < j; ++q)
+            if (q < (int)cnt && ns[q] == s[j]) { nk[q] |= k[j]; merged = true; }
+        if (merged) continue;
+#pragma unroll
+        for (int q = 0; q <= j; ++q)
+            if (q == (int)cnt) { ns[q] = s[j]; nk[q] = k[j]; }
+        ++cnt;
+    }
+#pragma unroll
+    for (int j = 0; j < kRuns; ++j) { s[j] = ns[j]; k[j] = nk[j]; }
+}
+
+struct HeadShared {
+    uint8_t text[kHeadChunks * kHeadStride];
+    uint32_t s[kRuns][kHeadChunks], k[kRuns][kHeadChunks], cnt[kHeadChunks], col[kHeadChunks];
+    uint16_t wide[kHeadChunks];              // chunks of this round with more than kRuns slots: slots << 8 | chunk
+    uint32_t pr[kHeadChunks], nwide;
+};
+
+// The chunk of slot q of a round, and where its staged window starts.
+template <bool FWD> struct HeadChunk {
+    uint64_t base;
+    uint32_t i, len, win;                    // window: bytes [win, win + kHeadWindow) of the chunk, inside it
+    __device__ HeadChunk(const Params &p, uint64_t first, uint32_t q) {
+        i = (uint32_t)(first + q);
+        base = (uint64_t)i * p.k;
+        len = chunk_len(p, i);
+        win = FWD || len <= kHeadWindow - 15 ? 0u : (len - (kHeadWindow - 15)) & ~15u;
+    }
+};
+
+// One byte, then four bytes of text, for the first W of a lane's runs.
+template <int W>
+__device__ __forceinline__ void head_byte(const LaneTab &T, uint32_t byte, uint32_t (&s)[kRuns]) {
+    const uint32_t col = lane_col<0>(T, byte);
+#pragma unroll
+    for (int j = 0; j < W; ++j) s[j] = lds8(s[j] * T.rowb + col);
+}
+template <bool FWD, int W>
+__device__ __forceinline__ void head_word(const LaneTab &T, uint32_t w, uint32_t (&s)[kRuns]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) head_byte<W>(T, __byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)), s);
+}
+
+// A round of a block: chunks first .. first + cnt - 1 (cnt <= per).
+template <bool FWD>
+__device__ void head_round(const Params &p, const LaneTab &T, HeadShared &S, uint64_t first, uint32_t cnt) {
+    const DevTables &t = p.t;
+    const uint32_t ms = FWD ? t.msf : t.msb;
+    const uint32_t *starts = FWD ? t.fSlotStart : t.bSlotStart;
+    if (threadIdx.x == 0) S.nwide = 0;
+    // text windows, 16 bytes a thread
+    for (uint32_t q = threadIdx.x; q < cnt * (kHeadWindow / 16); q += blockDim.x) {
+        const HeadChunk<FWD> c(p, first, q / (kHeadWindow / 16));
+        const uint32_t at = 16 * (q % (kHeadWindow / 16));
+        if (c.win + at < c.len) {
+            const uint4 v = load16(p.x, p.n, c.base + c.win + at);
+            uint32_t *d = reinterpret_cast<uint32_t *>(S.text + (q / (kHeadWindow / 16)) * kHeadStride + at);
+            d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+        }
+    }
+    __syncthreads();
+    // slots of each chunk
+    bool exact = false;
+    if (threadIdx.x < cnt) {
+        const uint32_t q = threadIdx.x;
+        const HeadChunk<FWD> c(p, first, q);
+        exact = FWD ? (c.i == 0 && !(p.shard & SHARD_PREV)) : (c.i == p.c - 1 && !(p.shard & SHARD_NEXT));
+        uint32_t m = 0;
+        if (!exact) {
+            const uint64_t e = FWD ? c.base : c.base + c.len;    // the edge
+            const uint32_t pr = __ldg(t.cls + __ldg(p.x + e - 1)) * t.ncls + __ldg(t.cls + __ldg(p.x + e));
+            m = __ldg((FWD ? t.fSlotCount : t.bSlotCount) + pr);
+            S.pr[q] = pr;
+            if (m > (uint32_t)kRuns) S.wide[atomicAdd(&S.nwide, 1u)] = (uint16_t)(m << 8 | q);
+            else
+                for (uint32_t j = 0; j < (uint32_t)kRuns; ++j) {
+                    S.s[j][q] = j < m ? __ldg(starts + (size_t)pr * ms + j) : 0u;
+                    S.k[j][q] = 1u << j;
+                }
+        }
+        S.cnt[q] = m > (uint32_t)kRuns ? 0u : m;
+        S.col[q] = FWD ? 1u : c.len - 1;                      // the slots' states include the edge byte
+    }
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31;
+    // chunks with more slots than a lane holds: a warp each, a lane per slot
+    for (uint32_t r = threadIdx.x >> 5; r < S.nwide; r += blockDim.x / 32) {
+        const uint32_t q = S.wide[r] & 0xFFu, m = S.wide[r] >> 8;
+        const HeadChunk<FWD> ch(p, first, q);
+        uint32_t v = lane < m ? __ldg(starts + (size_t)S.pr[q] * ms + lane) : 0u, c = FWD ? 1u : ch.len - 1;
+        for (;;) {
+            // to a multiple of four bytes, or the chunk's end
+            const uint32_t to = FWD ? min((c + 4) & ~3u, ch.len) : (c - 1) & ~3u;
+            while (c != to) {
+                const uint32_t at = FWD ? c : c - 1, w = at - ch.win;
+                v = lane_step<0>(T, v, w < kHeadWindow ? S.text[q * kHeadStride + w] : __ldg(p.x + ch.base + at));
+                c = FWD ? c + 1 : c - 1;
+            }
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, v);
+            const bool is_lead = v != 0 && lane == (uint32_t)__ffs(same) - 1;
+            const unsigned lead = __ballot_sync(0xFFFFFFFFu, is_lead);
+            const uint32_t n = __popc(lead);
+            if (n <= (uint32_t)kRuns) {
+                const uint32_t at = __popc(lead & ((1u << lane) - 1));
+                if (is_lead) { S.s[at][q] = v; S.k[at][q] = same; }
+                if (lane >= n && lane < (uint32_t)kRuns) { S.s[lane][q] = 0; S.k[lane][q] = 0; }
+                if (lane == 0) { S.cnt[q] = n; S.col[q] = c; }
+                break;
+            }
+            if (FWD ? c >= ch.len : c == 0) {                 // never met: every slot's end state
+                if (lane < ms) ((FWD ? p.w.Rf : p.w.Rb) + (size_t)ch.i * ms)[lane] = v;
+                if (lane == 0) { S.cnt[q] = kRuns + 1; S.col[q] = c; }
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    // a lane per chunk
+    if (threadIdx.x < ((cnt + 31) & ~31u)) {
+        const uint32_t q = threadIdx.x;
+        const bool valid = q < cnt;
+        const HeadChunk<FWD> ch(p, first, valid ? q : 0);
+        const uint32_t nU = (ch.len + kUnit - 1) / kUnit;
+        uint32_t s[kRuns], k[kRuns], n = 0, c = 0, conv = FWD ? 0 : nU, kind = 0;
+        bool open = false, all = false;                       // all: every slot's end state is written already
+#pragma unroll
+        for (int j = 0; j < kRuns; ++j) s[j] = k[j] = 0;
+        if (valid && exact) {                                 // J_0 = I, or F past the last chunk
+            s[0] = FWD ? t.fI : t.bF;
+            k[0] = 1;
+        } else if (valid) {
+            n = S.cnt[q];
+            c = S.col[q];
+            all = n > (uint32_t)kRuns;
+            open = !all && (FWD ? c < ch.len : c > 0);
+#pragma unroll
+            for (int j = 0; j < kRuns; ++j)
+                if (!all) { s[j] = S.s[j][q]; k[j] = S.k[j][q]; }
+            if (!open) {                                      // walked to the chunk's end
+                conv = FWD ? nU : 0;
+                kind = n > 1 ? 1u : 0u;
+            }
+        }
+        const uint8_t *text = S.text + q * kHeadStride;
+        while (__any_sync(0xFFFFFFFFu, open)) {
+            const uint32_t wm = __reduce_max_sync(0xFFFFFFFFu, open ? n : 0u);
+            if (open) {                                       // one unit, or what is left of it
+                const uint32_t to = FWD ? min((c / kUnit + 1) * kUnit, ch.len) : (c - 1) / kUnit * kUnit;
+                auto go = [&](auto width) {
+                    constexpr int Wd = decltype(width)::value;
+#pragma unroll 1
+                    while (c != to) {
+                        const uint32_t left = FWD ? to - c : c - to, at = FWD ? c : c - 1;
+                        if ((c & 3) == 0 && left >= 4) {      // four bytes
+                            const uint32_t a4 = FWD ? c : c - 4, w = a4 - ch.win;
+                            const uint32_t x = w < kHeadWindow ? *reinterpret_cast<const uint32_t *>(text + w)
+                                                               : __ldg(reinterpret_cast<const uint32_t *>(p.x + ch.base + a4));
+                            head_word<FWD, Wd>(T, x, s);
+                            c = FWD ? c + 4 : c - 4;
+                        } else {
+                            const uint32_t w = at - ch.win;
+                            head_byte<Wd>(T, w < kHeadWindow ? text[w] : __ldg(p.x + ch.base + at), s);
+                            c = FWD ? c + 1 : c - 1;
+                        }
+                    }
+                };
+                if (wm <= 1) go(std::integral_constant<int, 1>{});
+                else if (wm <= 2) go(std::integral_constant<int, 2>{});
+                else go(std::integral_constant<int, kRuns>{});
+                merge_runs(s, k, n);
+                const bool end = FWD ? c >= ch.len : c == 0;
+                if (n <= 1 || end) {
+                    open = false;
+                    conv = FWD ? (c + kUnit - 1) / kUnit : c / kUnit;
+                    kind = n > 1 ? 1u : 0u;
+                }
+            }
+        }
+        if (valid) {
+            if (kind && !all) {
+                uint32_t *R = (FWD ? p.w.Rf : p.w.Rb) + (size_t)ch.i * ms;
+                for (uint32_t j = 0; j < ms; ++j) {
+                    uint32_t v = 0;
+#pragma unroll
+                    for (int r = 0; r < kRuns; ++r)
+                        if ((k[r] >> j) & 1u) v = s[r];
+                    R[j] = v;
+                }
+            }
+            (FWD ? p.w.fconv : p.w.bconv)[ch.i] = conv;
+            (FWD ? p.w.fnrec : p.w.bnrec)[ch.i] = s[0];
+            (FWD ? p.w.fhit : p.w.bhit)[ch.i] = k[0];
+            (FWD ? p.w.fkind : p.w.bkind)[ch.i] = kind;
+        }
+    }
+    __syncthreads();                                          // S is refilled next
+}
+
+// Even blocks walk heads forward, odd ones backward (all forward for the
+// recognizer); a block stages its direction's table.
+__global__ void __launch_bounds__(kHeadThreads) heads_kernel(const __grid_constant__ Params p, uint32_t per) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ __align__(128) uint8_t cls[256];
+    __shared__ HeadShared S;
+    pdl_trigger();
+    if (blockIdx.x == 0) {                                    // the join's flags: read by the kernels after this one
+        if (threadIdx.x < FLAG_COUNT) p.w.flags[threadIdx.x] = threadIdx.x < 2 ? (int32_t)p.c : 0;
+        if (threadIdx.x >= 32 && threadIdx.x < 32 + kScanWords) p.w.scan[threadIdx.x - 32] = 0;
+    }
+    const bool pairs = !p.recognize, backward = pairs && (blockIdx.x & 1);
+    const uint32_t cw = class_words(p.t);
+    const LaneTab T{smem_u32(sm), cls, cw * 4};
+    stage_classes(p.t, cls);
+    stage_lane_table<0>(backward ? p.t.bc8 : p.t.fc8, (backward ? p.t.nb : p.t.nf) * cw, sm);
+    const uint64_t blk = pairs ? blockIdx.x >> 1 : blockIdx.x, nblk = pairs ? gridDim.x >> 1 : gridDim.x;
+    for (uint64_t first = blk * per; first < p.c; first += nblk * per) {   // head_round's first barrier: the tables are staged
+        const uint32_t cnt = (uint32_t)min((uint64_t)per, p.c - first);
+        if (backward) head_round<false>(p, T, S, first, cnt);
+        else head_round<true>(p, T, S, first, cnt);
+    }
+}
+
+}  // namespace
+
+// Chunks per block and round: kHeadChunks, fewer while that leaves the device
+// short of blocks (a warp takes about 1 us per chunk with many slots).
+void launch_heads(const Params &p, cudaStream_t s, int sm_count) {
+    const size_t smem = (size_t)std::max(p.t.nf, p.t.nb) * class_words(p.t) * 4;
+    static uint64_t attr_done = 0;
+    allow_smem(heads_kernel, &attr_done);
+    int per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, heads_kernel, kHeadThreads, smem);
+    const uint64_t dirs = p.recognize ? 1 : 2;
+    uint32_t per = kHeadChunks;
+    while (per > 8 && dirs * p.c / per < (uint64_t)sm_count * 2) per >>= 1;
+    const uint64_t want = (p.c + per - 1) / per, slots = (uint64_t)std::max(per_sm, 1) * sm_count / dirs;
+    heads_kernel<<<(uint32_t)(std::max<uint64_t>(1, std::min(want, slots)) * dirs), kHeadThreads, smem, s>>>(p, per);
+}
+
+}  // namespace slpf

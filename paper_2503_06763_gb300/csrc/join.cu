@@ -13,7 +13,7 @@
 // rejected (no accepting run: every clean column is empty).
 #include <algorithm>
 
-#include "kernels.cuh"
+#include "walk.cuh"
 
 namespace slpf {
 namespace {
@@ -343,10 +343,10 @@ __device__ void status_of(const Params &p) {
     if (ffail < (int32_t)p.c || (!p.recognize && bfail < (int32_t)p.c)) {
         st = RE_REJECTED;
     } else if (p.recognize) {
-        const uint32_t jc = p.w.FJ[p.c];
+        const uint32_t jc = __ldcg(p.w.FJ + p.c);
         if (!any_and(t.fBits + (size_t)jc * t.W, t.bBits + (size_t)t.bF * t.W, t.W)) st = RE_REJECTED;
     } else {
-        const uint32_t b0 = p.w.BJ[0];
+        const uint32_t b0 = __ldcg(p.w.BJ);
         if (!(b0 && any_and(t.fBits + (size_t)t.fI * t.W, t.bBits + (size_t)b0 * t.W, t.W))) st = RE_REJECTED;
     }
     if (__ldcg(&p.w.flags[FLAG_INTERNAL])) st = RE_E_INTERNAL;
@@ -452,8 +452,9 @@ __device__ uint32_t scan_step(const Params &p, uint32_t i, uint32_t cur) {
     return 1;
 }
 
+// False when a barrier wait ran out.
 template <uint32_t LANES>
-__device__ void join_scan(const Params &p) {
+__device__ bool join_scan(const Params &p) {
     const uint32_t lane = LANES == 1 ? 0u : (threadIdx.x & 31), upb = blockDim.x / LANES;
     const uint64_t gw = (uint64_t)blockIdx.x * upb + threadIdx.x / LANES, nw = (uint64_t)gridDim.x * upb;
     const bool bwd = !p.recognize;
@@ -475,8 +476,8 @@ __device__ void join_scan(const Params &p) {
         if (lane == 0) p.w.bLink[i] = p.w.bkind[i] ? (uint32_t)i + 1 : kResolved;
     }
     if (bad) atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
-    if (p.scan_stall && blockIdx.x == 0) return;      // test hook: the other blocks' waits run out
-    if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return; }
+    if (p.scan_stall && blockIdx.x == 0) return false;   // test hook: the other blocks' waits run out
+    if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return false; }
     for (uint32_t r = 0; r < kScanRounds; ++r) {
         uint32_t open = 0;
         for (uint64_t i = gw; i < p.c; i += nw) {
@@ -485,9 +486,10 @@ __device__ void join_scan(const Params &p) {
         }
         if (LANES == 1) open = __reduce_add_sync(0xFFFFFFFFu, open);
         if ((threadIdx.x & 31) == 0 && open) atomicAdd(p.w.scan + 2 + r, open);
-        if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return; }
+        if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return false; }
         if (__ldcg(p.w.scan + 2 + r) == 0) break;     // every chunk resolved (same value in every block)
     }
+    return true;
 }
 
 __global__ void __launch_bounds__(kBlockThreads) join_scan_kernel(const __grid_constant__ Params p) {
@@ -496,6 +498,70 @@ __global__ void __launch_bounds__(kBlockThreads) join_scan_kernel(const __grid_c
     if (__ldcg(p.w.scan + kScanGeneral) == 0 && !p.scan_stall) return;
     if (p.t.nfd < 16 && p.t.nbd < 16) join_scan<1>(p);   // tables of at most 16 entries: a thread per chunk
     else join_scan<32>(p);
+}
+
+// ------------------------------------------------------------------ after the lane walk
+// A general chunk (kind 1: its runs never met) of the lane walk, once the scan
+// has its output: the walk had no state to go on with, so the head of the
+// chunk its run enters is walked here, with the check the walk makes.
+template <bool FWD, bool OUT>
+__device__ void join_walk_fix(const Params &p, const LaneTab &T, uint32_t ns, uint32_t i) {
+    const uint32_t *kinds = FWD ? p.w.fkind : p.w.bkind, *J = FWD ? p.w.FJ : p.w.BJ;
+    if (!kinds[i]) return;
+    uint8_t *S = FWD ? p.w.FS : p.w.BS;
+    const uint32_t in = __ldcg(J + (FWD ? i : i + 1)), out = __ldcg(J + (FWD ? i + 1 : i));
+    bool fail = in == 0 || out == 0 || out >= ns;
+    if (OUT && FWD && i == p.c - 1) S[p.n] = (uint8_t)out;
+    if (!fail && (FWD ? i + 1 < p.c : i > 0)) {
+        const uint32_t o = FWD ? i + 1 : i - 1;
+        const uint64_t nbase = (uint64_t)o * p.k;
+        const uint32_t nlen = chunk_len(p, o), edge = min(kUnit * (FWD ? p.w.fconv : p.w.bconv)[o], nlen);
+        uint32_t mid;
+        const uint32_t e = walk_cols<0, FWD, OUT>(T, p.x, S, nbase + (FWD ? 0 : edge), nbase + (FWD ? edge : nlen),
+                                                  nbase + (FWD ? 0 : nlen), out,
+                                                  (reinterpret_cast<uintptr_t>(p.x) & 31) == 0, mid);
+        if (kinds[o] == 0) fail = e == 0 || e != (FWD ? p.w.fnrec : p.w.bnrec)[o];
+    }
+    if (fail) atomicMin(&p.w.flags[FWD ? FLAG_FFAIL : FLAG_BFAIL], (int32_t)i);
+}
+
+// The status after the lane walk.  The walk has checked every chunk whose
+// runs met (J_i is the state before it, and it enters live slots exactly when
+// the walk through the head reaches their state), so without general chunks
+// nothing is left but the verdict; with them, the scan over their maps, the
+// heads after them and then the verdict, separated by the bounded grid
+// barrier (cooperative launch).
+__global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_constant__ Params p) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    if (__ldcg(p.w.scan + kScanGeneral) == 0 && !p.scan_stall) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) status_of(p);
+        return;
+    }
+    const bool ok = p.t.nfd < 16 && p.t.nbd < 16 ? join_scan<1>(p) : join_scan<32>(p);
+    if (!ok) {
+        if (threadIdx.x == 0) atomicExch(p.status, RE_E_TIMEOUT);
+        return;
+    }
+    const uint32_t cw = class_words(p.t), nsf = p.t.nfd + 1, nsb = p.t.nbd + 1;
+    stage_classes(p.t, sm);
+    stage_lane_table<0>(p.t.fc8, nsf * cw, sm + 256);
+    stage_lane_table<0>(p.t.bc8, nsb * cw, sm + 256 + nsf * cw * 4);
+    __syncthreads();
+    const LaneTab F{smem_u32(sm + 256), sm, cw * 4}, B{smem_u32(sm + 256 + nsf * cw * 4), sm, cw * 4};
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.c; i += (uint64_t)gridDim.x * blockDim.x) {
+        if (p.mat) {
+            join_walk_fix<true, true>(p, F, nsf, (uint32_t)i);
+            join_walk_fix<false, true>(p, B, nsb, (uint32_t)i);
+        } else {
+            join_walk_fix<true, false>(p, F, nsf, (uint32_t)i);
+            if (!p.recognize) join_walk_fix<false, false>(p, B, nsb, (uint32_t)i);
+        }
+    }
+    if (!grid_barrier(p.w.scan)) {
+        if (threadIdx.x == 0) atomicExch(p.status, RE_E_TIMEOUT);
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) status_of(p);
 }
 
 // ------------------------------------------------------------------ batch
@@ -536,28 +602,34 @@ __global__ void batch_init_kernel(const Params *texts, uint32_t nt, uint32_t *qu
 
 }  // namespace
 
+// Cooperative launch of kernel with a warp (or a thread) per chunk, at most
+// the blocks the device holds at once.
+template <typename... KArgs, typename... Args>
+static bool launch_coop(void (*kernel)(KArgs...), size_t smem, uint64_t chunks, cudaStream_t s, int sm_count,
+                        Args &&...args) {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlockThreads, smem);
+    const uint64_t want = (chunks + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)std::max(per_sm, 1) * sm_count));
+    cfg.blockDim = kBlockThreads;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) == cudaSuccess;
+}
+
 // Classify, then the scan (a cooperative launch: its blocks meet at grid
 // barriers, so they must all be resident) or the chains, then verify.
 bool launch_join(const Params &p, cudaStream_t s, int sm_count) {
     const uint32_t blocks = (p.c + kBlockThreads - 1) / kBlockThreads;
     launch_dependent(join_classify_kernel, blocks, kBlockThreads, 0, s, p);
     if (p.scan) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, join_scan_kernel, kBlockThreads, 0);
-        const uint64_t units = p.c;                      // a warp (or a thread) per chunk and round
-        const uint64_t want = (units + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
-        const uint32_t grid = (uint32_t)std::max<uint64_t>(
-            1, std::min<uint64_t>(want, (uint64_t)std::max(per_sm, 1) * sm_count));
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = kBlockThreads;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, join_scan_kernel, p) != cudaSuccess) return false;
+        if (!launch_coop(join_scan_kernel, 0, p.c, s, sm_count, p)) return false;
     } else {
         launch_dependent(join_chain_kernel, blocks, kBlockThreads, 0, s, p);
     }
@@ -573,24 +645,17 @@ void launch_batch_init(const Params *texts, uint32_t nt, uint32_t *queues, uint3
     batch_init_kernel<<<(n + kBlockThreads - 1) / kBlockThreads, kBlockThreads, 0, s>>>(texts, nt, queues, nq);
 }
 
-// A slice's maps: classify (for the chunks' live slots), then the reduction.
+bool launch_join_walk(const Params &p, cudaStream_t s, int sm_count) {
+    const size_t smem = 256 + (size_t)(p.t.nfd + p.t.nbd + 2) * class_words(p.t) * 4;
+    static uint64_t attr_done = 0;
+    allow_smem(join_walk_kernel, &attr_done);
+    return launch_coop(join_walk_kernel, smem, p.c, s, sm_count, p);
+}
+
+// A slice's maps after the lane walk (every slot's end state, p.rall) or the
+// other reach shapes.
 bool launch_shard_map(const Params &p, uint8_t *d_maps, cudaStream_t s, int sm_count) {
-    const uint32_t blocks = (p.c + kBlockThreads - 1) / kBlockThreads;
-    launch_dependent(join_classify_kernel, blocks, kBlockThreads, 0, s, p);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, join_map_kernel, kBlockThreads, 0);
-    const uint64_t want = ((uint64_t)p.c + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
-    const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)std::max(per_sm, 1) * sm_count));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = kBlockThreads;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, join_map_kernel, p, d_maps) == cudaSuccess;
+    return launch_coop(join_map_kernel, 0, p.c, s, sm_count, p, d_maps);
 }
 
 void launch_join_batch(const BatchGroup &b, cudaStream_t s) {

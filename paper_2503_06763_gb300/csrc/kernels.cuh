@@ -46,8 +46,10 @@ struct Work {                       // device workspace, carved from the caller'
     uint32_t *FC, *BC;              // [Gc] checkpoints
     uint32_t *fconv, *bconv;        // [c] first / last sub-chunk boundary the reach runs agree on
     uint32_t *fkind, *bkind;        // [c] 0: every live slot ends in one state, 1: several
-    uint32_t *fnrec, *bnrec;        // [c] boundaries recorded (from the chunk's start / end)
-    uint32_t *fhit, *bhit;          // [c] slots the exact input state J_{i-1} / Ĵ_{i+1} enters
+    uint32_t *fnrec, *bnrec;        // [c] boundaries recorded (from the chunk's start / end); the lane
+                                    // walk: the state at the unit boundary fconv / bconv
+    uint32_t *fhit, *bhit;          // [c] slots the exact input state J_{i-1} / Ĵ_{i+1} enters; the lane
+                                    // walk: slots alive at that boundary
     uint32_t *recFc, *recBc;        // [c][kRecBounds] runs recorded at each boundary
     uint2 *recFe, *recBe;           // [c][kRecEntries] (state, slot set) of those runs
     int32_t *flags;                 // [FLAG_COUNT]
@@ -76,6 +78,7 @@ struct Params {
     uint32_t rvar;                  // reach shape (RE_PARSE_REACH): 1 byte tables, one direction per
                                     // block; 2 / 3 warp pairs, 3 / 2 stages; 4 one lane per chunk
     uint32_t rstages;               // TMA ring stages of the warp-pair and one-lane shapes
+    uint32_t rall;                  // the walk writes every slot's end state (slice maps), no columns
     uint32_t shard;                 // a slice of a longer text: SHARD_PREV, its first chunk speculates from
                                     // the byte before it (x[-1]); SHARD_NEXT, its last chunk from the
                                     // byte after it (x[len])
@@ -530,6 +533,11 @@ void launch_fixup_mat_batch(const BatchGroup &b, cudaStream_t s, int sm_count);
 void launch_gather_batch(const BatchGroup &b, const Params &like, cudaStream_t s, int sm_count);
 // Warps per direction of the byte-table reach (shape 1) on this device.
 uint64_t reach_byte8_warps(const Params &p, uint32_t ms, int sm_count);
+// The lane walk (heads.cu, walk.cu) and the join after it.
+void launch_heads(const Params &p, cudaStream_t s, int sm_count);
+void launch_walk(const Params &p, const CUtensorMap &text_map, const StateMaps &smaps, cudaStream_t s, int sm_count);
+uint64_t walk_lanes(const DevTables &t, bool recognize, int sm_count);
+bool launch_join_walk(const Params &p, cudaStream_t s, int sm_count);
 bool launch_join(const Params &p, cudaStream_t s, int sm_count);
 bool launch_shard_map(const Params &p, uint8_t *d_maps, cudaStream_t s, int sm_count);
 void launch_fixup(const Params &p, cudaStream_t s, int sm_count);

@@ -900,25 +900,21 @@ __global__ void __launch_bounds__(kFixupThreads) fixup_mat_batch_kernel(const __
     }
 }
 
-// Build & merge from the stored states: C_r = B_r ∩ B̂_r (Eq. merger) for
-// every column, encoded (DENSE bitset, or DICT index through the pair table
-// over classic-DFA state pairs).  A thread takes 16 consecutive columns: two
-// 16-byte state loads, 16 encoder lookups in shared memory, one vector store.
 // The gather's encoder over classic-DFA state pairs, staged in shared memory
-// (the caller synchronises): the DICT pair table, or the states' segment sets.
+// (the caller synchronises): the DICT pair table as 16-byte vectors of the
+// compiled copy (entry by entry from the 32-bit table of all states, a division
+// each, staging was most of a small text's gather: 34 us for 4 KB of log
+// text), or the states' segment sets.
 template <int E>
 __device__ Enc stage_gather_enc(const DevTables &t, uint8_t *sm) {
     const uint32_t nfs = t.nfd + 1, nbs = t.nbd + 1;
     Enc e{};
     e.nb = nbs;
     if constexpr (is_dict(E)) {
-        const size_t cnt = (size_t)nfs * nbs;
-        for (size_t q = threadIdx.x; q < cnt; q += blockDim.x) {
-            const uint32_t v = __ldg(t.pt + (q / nbs) * t.nb + q % nbs);
-            if (E == ENC_X1) sm[q] = (uint8_t)v;
-            else if (E == ENC_X2) reinterpret_cast<uint16_t *>(sm)[q] = (uint16_t)v;
-            else reinterpret_cast<uint32_t *>(sm)[q] = v;
-        }
+        const uint32_t cnt = (uint32_t)(((size_t)nfs * nbs * bytes_of(E) + 15) / 16);
+        const uint4 *src = reinterpret_cast<const uint4 *>(t.ptc);
+#pragma unroll 4
+        for (uint32_t q = threadIdx.x; q < cnt; q += blockDim.x) reinterpret_cast<uint4 *>(sm)[q] = __ldg(src + q);
         if (E == ENC_X1) e.pt8 = sm;
         else if (E == ENC_X2) e.pt16 = reinterpret_cast<uint16_t *>(sm);
         else e.pt32 = reinterpret_cast<uint32_t *>(sm);
@@ -1178,7 +1174,7 @@ void fixup_one(const Params &p, cudaStream_t s, int sm_count) {
 size_t gather_smem(const Params &p) {
     const size_t nfs = p.t.nfd + 1, nbs = p.t.nbd + 1;
     if (p.kind == RE_SLPF_PAIRS) return 0;
-    return p.kind == RE_SLPF_DICT ? nfs * nbs * p.col_bytes : (nfs + nbs) * 8;
+    return p.kind == RE_SLPF_DICT ? (nfs * nbs * p.col_bytes + 15) & ~(size_t)15 : (nfs + nbs) * 8;
 }
 
 template <int TM>

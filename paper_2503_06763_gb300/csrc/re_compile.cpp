@@ -864,9 +864,21 @@ re_status compile_pattern(const char *pattern, size_t len, const re_compile_opts
                     C.b2[(size_t)st * nc2 + c1 * ncls + c2] = mid | (C.bT[(size_t)mid * ncls + c1] << 16);
                 }
     }
+    // ---- the pair table over classic-DFA states, entries as wide as a DICT column
+    C.ptc.clear();
+    if (C.has_dict) {
+        const size_t nfs = C.nfd + 1, nbs = C.nbd + 1, cb = C.dict_size < 255 ? 1 : C.dict_size < 65535 ? 2 : 4;
+        C.ptc.assign((nfs * nbs * cb + 15) / 16 * 16, 0);
+        for (size_t f = 0; f < nfs; ++f)
+            for (size_t b = 0; b < nbs; ++b) {
+                const uint32_t v = C.pt[f * C.nb + b];
+                for (size_t q = 0; q < cb; ++q) C.ptc[(f * nbs + b) * cb + q] = (uint8_t)(v >> (8 * q));
+            }
+    }
     // ---- byte-indexed one-byte tables (states fit a byte): the reach looks a
     // transition up by the text byte itself, with no class lookup first.
     C.fbyte.clear(); C.bbyte.clear();
+    C.fc8.clear(); C.bc8.clear();
     if (C.nf <= 256 && C.nb <= 256) {
         C.fbyte.resize((size_t)C.nf * 256);
         C.bbyte.resize((size_t)C.nb * 256);
@@ -874,6 +886,14 @@ re_status compile_pattern(const char *pattern, size_t len, const re_compile_opts
             for (uint32_t b = 0; b < 256; ++b) C.fbyte[(size_t)st * 256 + b] = (uint8_t)C.fT[(size_t)st * ncls + C.cls[b]];
         for (uint32_t st = 0; st < C.nb; ++st)
             for (uint32_t b = 0; b < 256; ++b) C.bbyte[(size_t)st * 256 + b] = (uint8_t)C.bT[(size_t)st * ncls + C.cls[b]];
+        // class-indexed rows of whole words (the lane walk's tables)
+        const size_t row = 4 * ((size_t)(ncls + 3) / 4);
+        C.fc8.assign(C.nf * row, 0);
+        C.bc8.assign(C.nb * row, 0);
+        for (uint32_t st = 0; st < C.nf; ++st)
+            for (uint32_t c = 0; c < ncls; ++c) C.fc8[st * row + c] = (uint8_t)C.fT[(size_t)st * ncls + c];
+        for (uint32_t st = 0; st < C.nb; ++st)
+            for (uint32_t c = 0; c < ncls; ++c) C.bc8[st * row + c] = (uint8_t)C.bT[(size_t)st * ncls + c];
     }
     // ---- bytes 128..255 folded onto bytes below 128 of the same class: when
     // every class holding a byte >= 128 also holds one below, the byte-indexed

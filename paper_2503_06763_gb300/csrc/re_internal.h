@@ -53,8 +53,11 @@ struct DevTables {
     const uint8_t *bSlotOf;      // RE_COMPILE_DFA_STARTS_BWD only: [ncls][ncls][nb], the same backwards
     const uint32_t *pt;          // [nf][nb] dictionary index of B ∩ B̂ (DICT); pairs the
                                  // parse never produces hold 0xFFFFFFFF
+    const uint8_t *ptc;          // [nfd+1][nbd+1] the same over classic-DFA pairs, 1, 2 or 4 bytes an entry as
+                                 // the DICT columns (0xFF.. for the others); null without a dictionary
     const uint32_t *f2, *b2;     // [n][ncls^2] two-byte tables (mid | end << 16), or null
     const uint8_t *fbyte, *bbyte;  // [n][256] next state by byte (not class), u8; null unless n <= 256
+    const uint8_t *fc8, *bc8;    // [n][4 * ceil(ncls / 4)] next state by class, u8; null unless n <= 256
     const uint8_t *hirep;        // [128] byte b + 128 -> a byte below 128 of its class; null unless
                                  // every class holding a byte >= 128 holds one below (and fbyte is set)
     uint32_t fHashMask, bHashMask;
@@ -76,6 +79,7 @@ struct Compiled {
     std::vector<uint32_t> fT, bT;             // [n][ncls]
     std::vector<uint32_t> f2, b2;             // [n][ncls^2] two-byte tables (empty when too large)
     std::vector<uint8_t> fbyte, bbyte;        // [n][256] next state by byte (empty unless n <= 256)
+    std::vector<uint8_t> fc8, bc8;            // [n][4 * ceil(ncls / 4)] next state by class (empty unless n <= 256)
     std::vector<uint8_t> hirep;               // [128] representative below 128 of byte b + 128 (or empty)
     std::vector<uint64_t> fBits, bBits;       // [n][W]
     std::vector<uint32_t> fHash, bHash;
@@ -85,6 +89,7 @@ struct Compiled {
     std::vector<uint8_t> fSlotOf;             // RE_COMPILE_DFA_STARTS: [ncls][ncls][nf] slot of a state
     std::vector<uint8_t> bSlotOf;             // RE_COMPILE_DFA_STARTS_BWD: [ncls][ncls][nb] the same backwards
     std::vector<uint32_t> pt;                 // [nf][nb]
+    std::vector<uint8_t> ptc;                 // [nfd+1][nbd+1] the classic-DFA part, entries of the DICT column size
     std::vector<uint64_t> dict;               // [dict_size][W]
     uint32_t dict_size = 0;
     bool has_dict = false;
