@@ -793,6 +793,8 @@ extern "C" re_status re_matches(re_handle *h, const re_slpf *slpf, uint64_t len,
     a.col_bytes = cb;
     a.kind = kind;
     a.W = C.W;
+    a.ell = C.ell;
+    a.dict_size = C.dict_size;
     a.n = len;
     a.folseg = h->dev.folseg;
     a.dict = h->dev.dict;
@@ -802,7 +804,7 @@ extern "C" re_status re_matches(re_handle *h, const re_slpf *slpf, uint64_t len,
     a.pairs = d_pairs;
     a.cap = cap_pairs;
     a.count = d_count;
-    launch_matches(a, d_workspace, (cudaStream_t)stream);
+    launch_matches(a, d_workspace, (cudaStream_t)stream, sm_count_of(h->device));
     CUDA_TRY(cudaGetLastError(), "match launch");
     return RE_OK;
 }

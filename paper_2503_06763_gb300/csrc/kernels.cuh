@@ -549,15 +549,17 @@ constexpr int kMatchW = 8;                    // segment words supported (ell <=
 
 struct MatchArgs {
     const void *cols;                         // SLPF columns C_0 .. C_n
-    uint32_t col_bytes, kind, W;
+    uint32_t col_bytes, kind, W, ell, dict_size;
     uint64_t n;                               // text length (columns n + 1)
     const uint64_t *folseg;                   // [ell][W]
     const uint64_t *dict;                     // [dict_size][W] (DICT)
     const uint64_t *fbits, *bbits;            // [states][W] segment sets of the states (PAIRS)
     uint64_t open[kMatchW], close_first[kMatchW], whole[kMatchW], none[kMatchW];
     const int32_t *status;                    // parse status: anything but RE_OK gives no matches
-    uint64_t *cnt;                            // [G] pairs per warp range, then their exclusive offsets
+    uint64_t *cnt;                            // [G] pairs per tile, then their exclusive offsets
     uint64_t *bsum;                           // [ceil(G / kScanBlock)] block totals, then offsets
+    uint64_t *total;                          // [1] all matches
+    uint32_t *recs;                           // [G][kRecs] the count pass's spans of each tile
     uint64_t G;
     uint64_t *pairs;                          // [cap][2]
     uint64_t cap;
@@ -565,7 +567,7 @@ struct MatchArgs {
 };
 
 size_t match_workspace_bytes(uint64_t n);
-void launch_matches(MatchArgs a, void *ws, cudaStream_t s);
+void launch_matches(MatchArgs a, void *ws, cudaStream_t s, int sm_count);
 
 // Batch launchers: one launch per phase for every text of the group.
 void launch_batch_init(const Params *texts, uint32_t nt, uint32_t *queues, uint32_t nq, cudaStream_t s);
