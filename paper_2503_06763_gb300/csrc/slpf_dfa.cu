@@ -14,7 +14,8 @@
 // occurrence of (v, a) in the text.
 //
 // Encoding runs on the host (once per text, for storage); decoding is a
-// kernel with one thread per K-column piece.
+// kernel with one thread per K-column piece for short pieces, else a warp per
+// piece (slpf_dfa_warp_kernel).
 #include <algorithm>
 #include <cstring>
 #include <string>
@@ -161,6 +162,244 @@ __global__ void __launch_bounds__(256) slpf_dfa_decode_kernel(const __grid_const
     if (bad) atomicExch(a.status, RE_E_INTERNAL);
 }
 
+// Long pieces.  An exception is an exact column, so it is as good a place to
+// start from as a checkpoint: a warp takes a window of up to kWindow columns of
+// a piece and its lanes share it, lane j from the first exception at or after
+// column j * seg to the one where the next lane starts (the checkpoint for the
+// first).  Columns stand at 0.05 to 0.25 exceptions each, so the lanes' shares
+// are near seg, and a chain of dependent lookups is some 150 columns long
+// instead of K: for 48 MiB of log columns and K = 4096, where a thread per
+// piece left 12 289 chains of 4096 steps, the kernel went from 1371 to 138 us.
+//
+// In shared memory: the table, only the byte columns that occur (used bytes
+// renumbered; one byte per entry while ids and the mark of a missing entry
+// fit), the piece's exceptions, and a tile that holds each column's text byte
+// until the column replaces it.  The tile is padded by a word every 128 bytes,
+// as the lanes walk about 128 columns apart.  Bound by latency (the chains of
+// the longest share of each window) and issue: 16 warps a block 212 us, the 28
+// that the shared memory holds 138 us.
+constexpr uint32_t kWindow = 4096;
+template <int CB> constexpr uint32_t decode_warps() { return CB == 1 ? 28u : CB == 2 ? 16u : 8u; }   // what the shared memory holds
+constexpr uint32_t kDecodeExc = 512;           // exceptions staged per window; the rest are read from the archive
+constexpr uint32_t kDecodeTable = 48 * 1024;   // table bytes staged at most
+constexpr uint32_t kDecodeMinInterval = 256;
+
+template <int CB> struct IdOf;
+template <> struct IdOf<1> { using type = uint8_t; };
+template <> struct IdOf<2> { using type = uint16_t; };
+template <> struct IdOf<4> { using type = uint32_t; };
+
+template <int CB> __host__ __device__ constexpr uint32_t tile_at(uint32_t a) { return a * CB + (a * CB / 128) * 4; }
+template <int CB> __host__ __device__ constexpr uint32_t tile_bytes() { return (tile_at<CB>(kWindow) + 15) / 16 * 16; }
+
+template <int CB, bool BYTE>                   // BYTE: table entries of one byte (ids below 255)
+__global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kernel(const __grid_constant__ DecodeArgs a,
+                                                                          uint32_t table_bytes, uint32_t windows) {
+    using Id = typename IdOf<CB>::type;
+    using Entry = typename IdOf<BYTE ? 1 : 2>::type;
+    constexpr uint32_t none = BYTE ? 0xFFu : kNoEntry;
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ uint32_t used[256];
+    __shared__ uint8_t cls[256];               // byte -> column of the staged table
+    __shared__ uint32_t ncol;
+    // used byte columns: one entry of a row that occurs
+    for (uint32_t q = threadIdx.x; q < 256; q += blockDim.x) used[q] = 0;
+    __syncthreads();
+    const uint32_t rows = a.n_ids;
+    for (uint32_t q = threadIdx.x; q < rows * 128; q += blockDim.x) {
+        const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(a.table) + q);
+        if ((v & 0xFFFFu) != kNoEntry) used[2 * (q & 127)] = 1;
+        if (v >> 16 != kNoEntry) used[2 * (q & 127) + 1] = 1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        uint32_t n = 0;
+        for (uint32_t g = 0; g < 8; ++g) {
+            const uint32_t b = 32 * g + threadIdx.x;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, used[b] != 0);
+            cls[b] = (uint8_t)(n + __popc(m & ((1u << threadIdx.x) - 1)));
+            n += __popc(m);
+        }
+        if (threadIdx.x == 0) ncol = n;
+    }
+    __syncthreads();
+    // row stride: an odd number of words, so equal bytes of different rows are in different banks; the
+    // last column is that of every byte that does not occur
+    const uint32_t nc = ncol + 1;
+    const uint32_t rowe = ((nc * sizeof(Entry) + 3) / 4 | 1) * 4 / sizeof(Entry);
+    const bool staged = (uint64_t)rows * rowe * sizeof(Entry) <= table_bytes;
+    Entry *tab = reinterpret_cast<Entry *>(sm);
+    if (staged) {
+        for (uint32_t q = threadIdx.x; q < rows * 256; q += blockDim.x) {
+            const uint32_t b = q & 255, v = __ldg(a.table + q);
+            if (used[b]) tab[(q >> 8) * rowe + cls[b]] = v == kNoEntry ? (Entry)none : (Entry)v;
+        }
+        for (uint32_t q = threadIdx.x; q < rows; q += blockDim.x) tab[q * rowe + nc - 1] = (Entry)none;
+    }
+    __syncthreads();
+    if (threadIdx.x < 256 && !used[threadIdx.x]) cls[threadIdx.x] = (uint8_t)min(nc - 1, 255u);   // 256 used: no other byte
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint8_t *tile = sm + table_bytes + warp * (tile_bytes<CB>() + kDecodeExc * 4);
+    uint32_t *exc = reinterpret_cast<uint32_t *>(tile + tile_bytes<CB>());
+    Id *out = static_cast<Id *>(a.out);
+    auto next_of = [&](uint32_t cur, uint32_t byte) -> uint32_t {   // none: no such pair in the archived text
+        if (staged) return tab[cur * rowe + cls[byte]];
+        const uint32_t v = __ldg(a.table + (size_t)cur * 256 + byte);
+        return v == kNoEntry ? none : v;
+    };
+    bool bad = false;
+    for (uint64_t w = (uint64_t)blockIdx.x * decode_warps<CB>() + warp; w < a.n_checkpoints * windows;
+         w += (uint64_t)gridDim.x * decode_warps<CB>()) {
+        const uint64_t piece = w / windows, r0 = piece * a.interval;
+        const uint32_t len = (uint32_t)min((uint64_t)a.interval, a.n + 1 - r0), w0 = (uint32_t)(w % windows) * kWindow;
+        if (w0 >= len) continue;                              // the text's last piece is shorter
+        const uint32_t wl = min(kWindow, len - w0), seg = max(32u, (wl + 31) / 32);
+        const uint64_t e0 = __ldg(a.starts + piece), e1 = min(__ldg(a.starts + piece + 1), a.n_exceptions);
+        // first exception of [lo, hi) at or after column o of the piece
+        auto lower = [&](auto get, uint64_t lo, uint64_t hi, uint32_t o) -> uint64_t {
+            while (lo < hi) {
+                const uint64_t mid = (lo + hi) / 2;
+                if ((get(mid) >> 16) < o) lo = mid + 1; else hi = mid;
+            }
+            return lo;
+        };
+        auto global = [&](uint64_t e) -> uint32_t { return __ldg(a.exceptions + e); };
+        // none stands at the checkpoint column (a bad archive): the piece's start is the checkpoint
+        const uint64_t es = e0 < e1 ? lower(global, e0, e1, max(w0, 1u)) : e1;
+        __syncwarp();                                         // the last window's tile has left
+        for (uint32_t q = lane; q < kDecodeExc && es + q < e1; q += 32) exc[q] = __ldg(a.exceptions + es + q);
+        // text byte before each column: column c takes x[c - 1]
+        const bool vec = ((r0 + w0) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0;
+        const uint32_t wv = vec ? wl & ~15u : 0u;             // 16 columns a lane and turn
+        for (uint32_t q = 16 * lane; q < wv; q += 512) {
+            const uint8_t *at = a.x + r0 + w0 + q;
+            const uint4 v = load16(a.x, a.n, r0 + w0 + q);    // the text may end before the last column
+            const uint32_t before = r0 + w0 + q > 0 ? (uint32_t)__ldg(at - 1) : 0u;
+            const uint32_t w[5] = {before << 24, v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t four = __funnelshift_l(w[u], w[u + 1], 8);
+                uint32_t *d = reinterpret_cast<uint32_t *>(tile + tile_at<CB>(q + 4 * u));
+                if constexpr (CB == 1) {
+                    d[0] = four;
+                } else if constexpr (CB == 2) {
+                    d[0] = __byte_perm(four, 0u, 0x4140u);
+                    d[1] = __byte_perm(four, 0u, 0x4342u);
+                } else {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) d[b] = __byte_perm(four, 0u, 0x4440u | (uint32_t)b);
+                }
+            }
+        }
+        for (uint32_t q = wv + lane; q < wl; q += 32)
+            if (r0 + w0 + q > 0) *reinterpret_cast<Id *>(tile + tile_at<CB>(q)) = (Id)__ldg(a.x + r0 + w0 + q - 1);
+        __syncwarp();
+        auto get = [&](uint64_t e) -> uint32_t { return e - es < kDecodeExc ? exc[e - es] : __ldg(a.exceptions + e); };
+        // this lane's columns [from, to) of the piece
+        uint64_t e = lane == 0 && w0 == 0 ? es : lower(get, es, e1, w0 + lane * seg);
+        const uint64_t last = lower(global, es, e1, w0 + wl);
+        uint32_t ev = e < e1 ? get(e) : 0u;
+        uint32_t from = lane == 0 && w0 == 0 ? 0u : e < e1 ? ev >> 16 : len;
+        uint32_t to = __shfl_down_sync(0xFFFFFFFFu, from, 1);
+        if (lane == 31) to = last < e1 ? global(last) >> 16 : len;
+        from = min(from, len);
+        to = min(to, len);
+        const uint32_t first = __shfl_sync(0xFFFFFFFFu, from, 0);   // columns before it are the last window's
+        if (from < to) {
+            uint32_t cur;
+            if (lane == 0 && w0 == 0) {
+                cur = __ldg(a.checkpoints + piece);
+            } else {
+                cur = ev & 0xFFFFu;
+                ++e;
+                ev = e < e1 ? get(e) : 0u;
+            }
+            uint32_t next = e < e1 ? ev >> 16 : 0xFFFFFFFFu;
+            auto step = [&](uint32_t o, uint32_t byte) {      // column o of the piece from the one before
+                if (o == next) {
+                    cur = ev & 0xFFFFu;
+                    ++e;
+                    ev = e < e1 ? get(e) : 0u;
+                    next = e < e1 ? ev >> 16 : 0xFFFFFFFFu;
+                } else {
+                    const uint32_t v = cur < rows ? next_of(cur, byte) : none;
+                    bad |= v == none;                          // not an archive of this text
+                    cur = v == none ? 0u : v;
+                }
+            };
+            const uint32_t in = min(to, w0 + wl);             // columns inside the tile
+            uint32_t o = from;
+            if (o < in) { *reinterpret_cast<Id *>(tile + tile_at<CB>(o - w0)) = (Id)cur; ++o; }
+            else { out[r0 + o] = (Id)cur; ++o; }              // the share starts after the window
+            if (staged && e1 - es <= kDecodeExc) {            // the common case, on shared memory alone
+                uint32_t ei = (uint32_t)(e - es);
+                const uint32_t en = (uint32_t)(e1 - es);
+#pragma unroll 2
+                for (; o < in; ++o) {
+                    Id *t = reinterpret_cast<Id *>(tile + tile_at<CB>(o - w0));
+                    const uint32_t v = cur < rows ? (uint32_t)tab[cur * rowe + cls[(uint32_t)*t & 0xFFu]] : none;
+                    if (o == next) {
+                        cur = ev & 0xFFFFu;
+                        ++ei;
+                        ev = exc[min(ei, kDecodeExc - 1)];
+                        next = ei < en ? ev >> 16 : 0xFFFFFFFFu;
+                    } else {
+                        bad |= v == none;
+                        cur = v == none ? 0u : v;
+                    }
+                    *t = (Id)cur;
+                }
+                e = es + ei;
+            }
+            for (; o < in; ++o) {
+                Id *t = reinterpret_cast<Id *>(tile + tile_at<CB>(o - w0));
+                step(o, (uint32_t)*t & 0xFFu);
+                *t = (Id)cur;
+            }
+            for (; o < to; ++o) {
+                step(o, __ldg(a.x + r0 + o - 1));
+                out[r0 + o] = (Id)cur;
+            }
+        }
+        __syncwarp();
+        // the tile's columns out, from `first` on
+        constexpr uint32_t V = 4 / CB;                        // columns per word
+        const uint64_t c0 = r0 + w0;
+        const uint32_t skip = first > w0 ? min(first - w0, wl) : 0u;
+        constexpr uint32_t C16 = 4 * V;                       // columns per 16 bytes
+        if ((c0 % C16) == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15) == 0) {
+            for (uint32_t q = C16 * lane; q < wl; q += 32 * C16) {
+                if (q >= skip && q + C16 <= wl) {             // inside a 128-byte row of the tile
+                    const uint32_t *t = reinterpret_cast<const uint32_t *>(tile + tile_at<CB>(q));
+                    reinterpret_cast<uint4 *>(out)[(c0 + q) / C16] = make_uint4(t[0], t[1], t[2], t[3]);
+                } else {
+                    for (uint32_t u = 0; u < C16; ++u)
+                        if (q + u >= skip && q + u < wl) out[c0 + q + u] = *reinterpret_cast<const Id *>(tile + tile_at<CB>(q + u));
+                }
+            }
+        } else {
+            for (uint32_t q = skip + lane; q < wl; q += 32) out[c0 + q] = *reinterpret_cast<const Id *>(tile + tile_at<CB>(q));
+        }
+    }
+    if (bad) atomicExch(a.status, RE_E_INTERNAL);
+}
+
+template <int CB, bool BYTE>
+cudaError_t launch_decode_warp(const DecodeArgs &a, cudaStream_t s, int sms) {
+    const uint32_t windows = (a.interval + kWindow - 1) / kWindow;
+    const uint32_t table = std::min<uint32_t>(kDecodeTable, (uint32_t)(((size_t)a.n_ids * (260 + 4) * (BYTE ? 1 : 2) + 15) / 16 * 16));
+    const size_t smem = table + decode_warps<CB>() * (tile_bytes<CB>() + kDecodeExc * 4);
+    const cudaError_t e = cudaFuncSetAttribute(slpf_dfa_warp_kernel<CB, BYTE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slpf_dfa_warp_kernel<CB, BYTE>, decode_warps<CB>() * 32, smem);
+    const uint64_t want = (a.n_checkpoints * windows + decode_warps<CB>() - 1) / decode_warps<CB>();
+    const uint32_t blocks = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * std::max(per_sm, 1)));
+    slpf_dfa_warp_kernel<CB, BYTE><<<blocks, decode_warps<CB>() * 32, smem, s>>>(a, table, windows);
+    return cudaGetLastError();
+}
+
 __global__ void slpf_dfa_status_kernel(int32_t *status) { *status = RE_OK; }
 
 }  // namespace
@@ -259,6 +498,14 @@ extern "C" re_status re_slpf_dfa_decode(const re_slpf_dfa_header *hdr, const voi
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (hdr->interval >= kDecodeMinInterval) {                 // a warp per piece
+        cudaError_t e;
+        if (col_bytes == 1) e = hdr->n_ids < 255 ? launch_decode_warp<1, true>(a, s, sms) : launch_decode_warp<1, false>(a, s, sms);
+        else if (col_bytes == 2) e = hdr->n_ids < 255 ? launch_decode_warp<2, true>(a, s, sms) : launch_decode_warp<2, false>(a, s, sms);
+        else e = hdr->n_ids < 255 ? launch_decode_warp<4, true>(a, s, sms) : launch_decode_warp<4, false>(a, s, sms);
+        if (e != cudaSuccess) { set_error(std::string("decode launch: ") + cudaGetErrorString(e)); return RE_E_CUDA; }
+        return RE_OK;
+    }
     const uint64_t want = (hdr->n_checkpoints + 255) / 256;
     const uint32_t blocks = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 4));
     slpf_dfa_decode_kernel<<<blocks, 256, smem, s>>>(a);
