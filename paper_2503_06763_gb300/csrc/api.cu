@@ -54,6 +54,13 @@ int sm_count_of(int device) {
 bool walks(const re_handle *h);
 uint32_t table_mode(const DevTables &t);
 
+// n bytes over `target` chunks.
+uint32_t chunk_for(uint64_t n, uint64_t target) {
+    uint64_t k = (n + target - 1) / target;
+    k = (k + kSub - 1) / kSub * kSub;
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(k, 256), 1u << 20);
+}
+
 // Chunk length k.  Lane walk: a lane per chunk, as many chunks as the device
 // walks at once in a direction.  Otherwise one reach thread per chunk, about 2
 // resident warps per scheduler, chunks long enough that speculative runs meet
@@ -61,10 +68,7 @@ uint32_t table_mode(const DevTables &t);
 uint32_t choose_chunk(const re_handle *h, uint64_t n, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
     const bool rec = opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY);
-    const uint64_t target = walks(h) && table_mode(h->dev) == TM_SMEM ? walk_lanes(h->dev, rec, sms) : (uint64_t)sms * 384;
-    uint64_t k = (n + target - 1) / target;
-    k = (k + kSub - 1) / kSub * kSub;
-    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(k, 256), 1u << 20);
+    return chunk_for(n, walks(h) && table_mode(h->dev) == TM_SMEM ? walk_lanes(h->dev, rec, sms) : (uint64_t)sms * 384);
 }
 
 int length_bucket(uint64_t n) {
@@ -159,12 +163,11 @@ bool scan_join(const re_handle *h) { return h->host.nfd + 1 <= kScanStates && h-
 uint32_t table_mode(const DevTables &t);
 
 // Per-position states (mat): automata of at most 256 states per direction
-// (the byte tables exist, and every classic-DFA state fits a byte).
+// (every state fits a byte).
 bool mat_capable(const re_handle *h) {
-    const Compiled &C = h->host;
-    return !h->host_only && !C.fbyte.empty() && C.nf <= 256 && C.nb <= 256;
+    return !h->host_only && walks(h);
 }
-// Shapes whose reach kernels store the states: byte tables, or warp pairs
+// Shapes whose reach kernels store the states: the lane walk, or warp pairs
 // with u8 class tables (not the pair layout of small class alphabets).
 bool shape_stores_states(const re_handle *h, uint32_t v) {
     return v == 1 || ((v == 2 || v == 3) && table_mode(h->dev) == TM_SMEM);
@@ -330,9 +333,7 @@ re_status re_compile(const char *pattern, size_t len, const re_compile_opts *opt
     const size_t i_fs = add(C.folseg.data(), C.folseg.size() * 8), i_dc = add(C.dict.data(), C.dict.size() * 8);
     const size_t i_fso = add(C.fSlotOf.data(), C.fSlotOf.size());
     const size_t i_bso = add(C.bSlotOf.data(), C.bSlotOf.size());
-    const size_t i_fby = add(C.fbyte.data(), C.fbyte.size()), i_bby = add(C.bbyte.data(), C.bbyte.size());
     const size_t i_fc8 = add(C.fc8.data(), C.fc8.size()), i_bc8 = add(C.bc8.data(), C.bc8.size());
-    const size_t i_hr = add(C.hirep.data(), C.hirep.size());
     DevTables &t = h->dev;
     t.fHashMask = C.fHashMask; t.bHashMask = C.bHashMask;
     t.ncls = C.ncls; t.W = C.W; t.ell = C.ell;
@@ -365,11 +366,8 @@ re_status re_compile(const char *pattern, size_t len, const re_compile_opts *opt
     t.f2 = C.f2.empty() ? nullptr : (const uint32_t *)(b + pc[i_f2].off);
     t.b2 = C.b2.empty() ? nullptr : (const uint32_t *)(b + pc[i_b2].off);
     t.folseg = (const uint64_t *)(b + pc[i_fs].off);
-    t.fbyte = C.fbyte.empty() ? nullptr : b + pc[i_fby].off;
-    t.bbyte = C.bbyte.empty() ? nullptr : b + pc[i_bby].off;
     t.fc8 = C.fc8.empty() ? nullptr : b + pc[i_fc8].off;
     t.bc8 = C.bc8.empty() ? nullptr : b + pc[i_bc8].off;
-    t.hirep = C.hirep.empty() ? nullptr : b + pc[i_hr].off;
     t.dict = C.dict.empty() ? nullptr : (const uint64_t *)(b + pc[i_dc].off);
     *out = h;
     return RE_OK;
@@ -392,7 +390,7 @@ re_status re_get_info(const re_handle *h, re_info *info) {
     info->dict_size = C.has_dict ? C.dict_size : 0;
     info->inf_ambiguous = C.inf_amb ? 1u : 0u;
     info->sample_limit = C.sample_limit;
-    info->ascii_rows = C.hirep.empty() ? 0u : 1u;
+    info->ascii_rows = C.ascii_rows ? 1u : 0u;
     info->reach_shapes = shapes_of(h);
     return RE_OK;
 }
@@ -875,7 +873,8 @@ struct re_batch {
     struct Group {
         re_handle *h = nullptr;
         uint32_t tmode = 0, ms = 0, enc_in_smem = 0, cb = 1;
-        bool mat = false;               // per-position states (byte-table reach, fix-up of heads, gather)
+        bool walk = false;              // the lane walk (with per-position states unless recognizing)
+        uint32_t per = 0, logr = 0;     // heads round, table copies of the walk
         re_slpf_kind kind = RE_SLPF_DENSE;
         std::vector<uint32_t> members;  // caller indices, longest chunks first
         size_t params_off = 0, cbase_off = 0, rbase_off = 0, mbase_off = 0;
@@ -886,6 +885,10 @@ struct re_batch {
     std::vector<Text> texts;
     std::vector<Group> groups;
     size_t queue_off = 0, maps_off = 0, desc_bytes = 0, total = 0;
+    // lane-walk groups: their descriptors, and the group of each block of a phase
+    size_t wgroups_off = 0, heads_off = 0, walk_off = 0, gather_off = 0;
+    std::vector<slpf::WalkSpan> heads, walk, gather;
+    slpf::WalkBatch wb{};
     uint8_t *pinned = nullptr;
     cudaEvent_t uploaded = nullptr;
     bool pending = false;
@@ -909,14 +912,18 @@ struct re_batch {
 namespace slpf {
 namespace {
 
-// Chunk length of one text of a batch: the single-text rule applied to the
-// group's total bytes (one reach lane per chunk, about one wave of lanes for
-// the whole group), but short enough that the text spans a warp tile of 32
-// chunks where it can.
-uint32_t batch_chunk(const re_handle *h, uint64_t len, uint64_t group_bytes, int sms, const re_parse_opts *opts) {
+// Chunk length of one text of a batch.  Lane walk: the bytes of all its groups
+// over twice the lanes of a direction (a warp then takes about two tiles from
+// the queue), and a length that makes the text's chunks whole tiles of 32.
+// Otherwise the single-text rule applied to the group's total bytes (one reach
+// lane per chunk, about one wave of lanes for the whole group), but short
+// enough that the text spans a warp tile of 32 chunks where it can.
+uint32_t batch_chunk(const re_handle *h, uint64_t len, uint64_t group_bytes, bool walk, bool recognize, int sms,
+                     const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
-    const uint32_t kg = choose_chunk(h, group_bytes, sms, nullptr);
-    uint64_t kt = (len + 31) / 32;
+    const uint64_t kg = chunk_for(group_bytes, walk ? 2 * walk_lanes(h->dev, recognize, sms) : (uint64_t)sms * 384);
+    const uint64_t tiles = walk ? std::max<uint64_t>(1, (len + 32 * kg - 1) / (32 * kg)) : 1;
+    uint64_t kt = (len + 32 * tiles - 1) / (32 * tiles);
     kt = (kt + kSub - 1) / kSub * kSub;
     return (uint32_t)std::max<uint64_t>(256, std::min<uint64_t>(kg, kt));
 }
@@ -929,8 +936,83 @@ Params group_like(const re_batch::Group &g, bool recognize) {
     q.col_bytes = g.cb;
     q.recognize = recognize ? 1u : 0u;
     q.enc_in_smem = g.enc_in_smem;
-    q.mat = g.mat ? 1u : 0u;
+    q.mat = g.walk && !recognize ? 1u : 0u;
     return q;
+}
+
+// Blocks for each weight, about `budget` in all and at least one each, at most
+// cap[j]: by share, then the rest to whoever has the most per block.
+std::vector<uint32_t> share_blocks(const std::vector<uint64_t> &weight, const std::vector<uint64_t> &cap, uint64_t budget) {
+    uint64_t sum = 0, used = 0;
+    for (uint64_t w : weight) sum += w;
+    std::vector<uint32_t> out(weight.size(), 0);
+    for (size_t j = 0; j < weight.size(); ++j) {
+        if (!cap[j]) continue;
+        out[j] = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(cap[j], sum ? (uint64_t)((double)budget * weight[j] / sum) : 1));
+        used += out[j];
+    }
+    for (; used < budget; ++used) {
+        size_t best = weight.size();
+        for (size_t j = 0; j < weight.size(); ++j)
+            if (out[j] && out[j] < cap[j] &&
+                (best == weight.size() || (double)weight[j] / out[j] > (double)weight[best] / out[best])) best = j;
+        if (best == weight.size()) break;
+        ++out[best];
+    }
+    return out;
+}
+
+// A span per block of a phase.
+std::vector<WalkSpan> spans_of(const std::vector<uint32_t> &blocks) {
+    std::vector<WalkSpan> v;
+    for (uint32_t j = 0; j < blocks.size(); ++j)
+        for (uint32_t q = 0; q < blocks[j]; ++q) v.push_back(WalkSpan{j, q, blocks[j]});
+    return v;
+}
+
+// The launches of the lane-walk groups: how many blocks each group gets in
+// each phase (heads by chunks, walk by text bytes, gather by columns).
+void plan_walk(re_batch *b, const std::vector<uint64_t> &gbytes) {
+    const size_t ng = b->groups.size();
+    std::vector<uint64_t> chunks(ng, 0), tiles(ng, 0), mtiles(ng, 0), bytes(ng, 0), rounds(ng, 0);
+    uint64_t all = 0;
+    const uint64_t dirs = b->recognize ? 1 : 2;
+    WalkBatch &w = b->wb;
+    w.recognize = b->recognize ? 1u : 0u;
+    for (size_t j = 0; j < ng; ++j) {
+        const re_batch::Group &g = b->groups[j];
+        if (!g.walk) continue;
+        chunks[j] = g.chunks; tiles[j] = g.n_reach; mtiles[j] = g.n_merge; bytes[j] = gbytes[j];
+        all += g.chunks;
+        w.heads_smem = std::max(w.heads_smem, heads_smem(g.h->dev));
+        w.join_smem = std::max(w.join_smem, join_walk_smem(g.h->dev));
+        if (!b->recognize) w.gather_smem = std::max(w.gather_smem, mat_gather_smem(group_like(g, false)));
+    }
+    if (!all) return;                                         // no such group, or empty texts alone
+    uint32_t per = 64;
+    while (per > 8 && dirs * all / per < (uint64_t)b->sms * 2) per >>= 1;
+    for (size_t j = 0; j < ng; ++j) {
+        b->groups[j].per = per;
+        rounds[j] = (chunks[j] + per - 1) / per;
+    }
+    b->heads = spans_of(share_blocks(chunks, rounds, (uint64_t)b->sms * heads_blocks_per_sm(w.heads_smem) / dirs));
+    const std::vector<uint32_t> wblk = share_blocks(bytes, tiles, b->sms / dirs);
+    b->walk = spans_of(wblk);
+    for (size_t j = 0; j < ng; ++j) {
+        re_batch::Group &g = b->groups[j];
+        if (!wblk[j]) continue;
+        g.logr = (uint32_t)walk_copies(g.h->dev, tiles[j], wblk[j]);
+        w.walk_smem = std::max(w.walk_smem, walk_smem_bytes(g.h->dev, (int)g.logr));
+    }
+    if (!b->recognize) {
+        std::vector<uint64_t> cap(ng, 0);
+        for (size_t j = 0; j < ng; ++j) cap[j] = (mtiles[j] + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
+        const uint64_t per_sm = std::max<uint64_t>(1, std::min<uint64_t>(8, 200 * 1024 / (w.gather_smem + 1024)));
+        b->gather = spans_of(share_blocks(mtiles, cap, b->sms * per_sm));
+    }
+    w.n_heads = (uint32_t)b->heads.size();
+    w.n_walk = (uint32_t)b->walk.size();
+    w.n_gather = (uint32_t)b->gather.size();
 }
 
 re_status batch_run(re_batch *b, cudaStream_t s0) {
@@ -942,9 +1024,19 @@ re_status batch_run(re_batch *b, cudaStream_t s0) {
         CUDA_TRY(cudaEventRecord(b->fork, s0), "batch fork");
         for (cudaStream_t a : b->aux) CUDA_TRY(cudaStreamWaitEvent(a, b->fork, 0), "batch fork");
     }
+    bool walk = false;
+    for (const re_batch::Group &g : b->groups) walk = walk || g.walk;
+    if (walk) {                                               // one launch per phase over all these groups
+        launch_heads_batch(b->wb, s0);
+        launch_walk_batch(b->wb, s0);
+        launch_join_walk_batch(b->wb, s0);
+        launch_gather_batch(b->wb, s0);
+    }
+    size_t other = 0;
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         const re_batch::Group &g = b->groups[gi];
-        const cudaStream_t s = na ? b->aux[gi % na] : s0;
+        if (g.walk) continue;
+        const cudaStream_t s = na ? b->aux[other++ % na] : s0;
         BatchGroup bg{};
         bg.t = g.h->dev;
         bg.texts = reinterpret_cast<const Params *>(w + g.params_off);
@@ -955,16 +1047,6 @@ re_status batch_run(re_batch *b, cudaStream_t s0) {
         bg.chunks = g.chunks; bg.n_reach = g.n_reach; bg.n_merge = g.n_merge;
         bg.nt = (uint32_t)g.members.size();
         bg.recognize = b->recognize ? 1u : 0u;
-        if (g.mat) {
-            if (g.n_reach && !launch_reach_batch_byte8(bg, g.ms, s, b->sms)) {
-                set_error("too many speculative starts");
-                return RE_E_INTERNAL;
-            }
-            launch_join_batch(bg, s);
-            launch_fixup_mat_batch(bg, s, b->sms);
-            launch_gather_batch(bg, group_like(g, b->recognize), s, b->sms);
-            continue;
-        }
         if (g.n_reach && !launch_reach_batch(bg, g.tmode, g.ms, s, b->sms)) {
             set_error("too many speculative starts");
             return RE_E_INTERNAL;
@@ -1018,13 +1100,13 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
             g.h = h;
             g.tmode = table_mode(h->dev);
             g.ms = std::max(h->host.msf, b->recognize ? 1u : h->host.msb);
-            // per-position states where the single-text parse would use them (byte
-            // tables for both automata) and the slots fit the byte-table reach
-            g.mat = !b->recognize && mat_capable(h) && g.ms <= 32;
             if (!b->recognize) {
                 const re_status st = resolve_kind(h, opts ? opts->kind : RE_SLPF_AUTO, g.kind, g.cb);
                 if (st != RE_OK) return st;
             }
+            // the lane walk wherever the automata have byte states, as long as
+            // the gather's encoder fits shared memory
+            g.walk = walks(h) && (b->recognize || mat_gather_smem(group_like(g, false)) <= kSmemMergeMax);
             b->groups.push_back(std::move(g));
             gbytes.push_back(0);
         }
@@ -1033,12 +1115,15 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
         b->groups[it->second].members.push_back(j);
         gbytes[it->second] += lens[j];
     }
+    uint64_t walk_bytes = 0;                                 // the lane-walk groups run at once
+    for (size_t j = 0; j < b->groups.size(); ++j) walk_bytes += b->groups[j].walk ? gbytes[j] : 0;
     // chunk lengths, then members longest chunks first
     for (uint32_t j = 0; j < count; ++j) {
         re_batch::Text &t = b->texts[j];
-        t.k = batch_chunk(b->groups[t.group].h, t.len, gbytes[t.group], b->sms, opts);
+        const re_batch::Group &tg = b->groups[t.group];
+        t.k = batch_chunk(tg.h, t.len, tg.walk ? walk_bytes : gbytes[t.group], tg.walk, b->recognize, b->sms, opts);
         if (t.len / t.k >= 0xFFFFFFF0ull) { set_error("text too long for this chunk length"); return RE_E_INVALID_ARG; }
-        if (t.len) t.L = layout_for(b->groups[t.group].h, t.len, t.k, b->groups[t.group].mat);
+        if (t.len) t.L = layout_for(b->groups[t.group].h, t.len, t.k, mat_capable(tg.h) && !b->recognize);
     }
     uint32_t slot = 0;                                       // every text's Params, group after group
     for (auto &g : b->groups) {
@@ -1063,6 +1148,24 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
     }
     b->queue_off = off;
     off = align256(off + b->groups.size() * kQueues * sizeof(uint32_t));
+    for (auto &g : b->groups) {                              // units of each kind
+        for (uint32_t j : g.members) {
+            const re_batch::Text &t = b->texts[j];
+            const uint64_t c = t.len ? t.L.c : 0;
+            g.chunks += c;
+            g.n_reach += (c + 31) / 32;
+            g.n_merge += ((t.len && !b->recognize ? t.L.Gc : 0) + 31) / 32;
+        }
+        if (g.n_reach >= 0xFFFFFFFFull || g.n_merge >= 0xFFFFFFFFull) {
+            set_error("batch too large for one launch per phase");
+            return RE_E_INVALID_ARG;
+        }
+    }
+    plan_walk(b.get(), gbytes);
+    b->wgroups_off = off; off = align256(off + b->groups.size() * sizeof(WalkGroup));
+    b->heads_off = off; off = align256(off + b->heads.size() * sizeof(WalkSpan));
+    b->walk_off = off; off = align256(off + b->walk.size() * sizeof(WalkSpan));
+    b->gather_off = off; off = align256(off + b->gather.size() * sizeof(WalkSpan));
     b->desc_bytes = off;
     for (uint32_t j = 0; j < count; ++j) {
         re_batch::Text &t = b->texts[j];
@@ -1086,19 +1189,17 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
             rb[m + 1] = rb[m] + (c + 31) / 32;
             mb[m + 1] = mb[m] + (groups + 31) / 32;
         }
-        g.chunks = cb[g.members.size()];
-        g.n_reach = rb[g.members.size()];
-        g.n_merge = mb[g.members.size()];
-        if (g.n_reach >= 0xFFFFFFFFull || g.n_merge >= 0xFFFFFFFFull) {
-            set_error("batch too large for one launch per phase");
-            return RE_E_INVALID_ARG;
-        }
     }
+    if (!b->heads.empty()) std::memcpy(b->pinned + b->heads_off, b->heads.data(), b->heads.size() * sizeof(WalkSpan));
+    if (!b->walk.empty()) std::memcpy(b->pinned + b->walk_off, b->walk.data(), b->walk.size() * sizeof(WalkSpan));
+    if (!b->gather.empty()) std::memcpy(b->pinned + b->gather_off, b->gather.data(), b->gather.size() * sizeof(WalkSpan));
     CUDA_TRY(cudaEventCreateWithFlags(&b->uploaded, cudaEventDisableTiming), "batch event");
     uint64_t all_bytes = 0;
-    for (uint64_t g : gbytes) all_bytes += g;
-    if (b->groups.size() > 1 && all_bytes >= (64ull << 20)) {   // small batches: no stream set-up cost
-        const size_t na = std::min<size_t>(4, b->groups.size());
+    size_t others = 0;                                       // groups of the other kernels: a launch each
+    for (size_t j = 0; j < b->groups.size(); ++j)
+        if (!b->groups[j].walk) { all_bytes += gbytes[j]; ++others; }
+    if (others > 1 && all_bytes >= (64ull << 20)) {   // small batches: no stream set-up cost
+        const size_t na = std::min<size_t>(4, others);
         CUDA_TRY(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "batch event");
         for (size_t a = 0; a < na; ++a) {
             cudaStream_t st;
@@ -1164,18 +1265,44 @@ re_status re_parse_batch(re_batch *b, const uint8_t *const *d_texts, re_slpf *ou
         p.Gfast = t.len / kSub;
         p.c_full = (uint32_t)(t.len / t.k);
         if (t.len) carve(p, t.L, w + t.ws_off);
-        if (g.mat && t.len) {                                // TMA for full tiles: maps in the descriptor area
+        if (g.walk) {
+            p.rvar = 1;
+            p.scan = 1;
+        }
+        if (g.walk && t.len) {                               // TMA for full tiles: maps in the descriptor area
             CUtensorMap *hm = reinterpret_cast<CUtensorMap *>(b->pinned + b->maps_off) + 3 * (size_t)t.slot;
             uint8_t *ws = w + t.ws_off;
-            p.text_tma = text_tensor_map(hm[0], d_texts[j], t.k, p.c_full) &&
-                         text_tensor_map(hm[1], ws + t.L.off[24], t.k, p.c_full) &&
-                         text_tensor_map(hm[2], ws + t.L.off[25], t.k, p.c_full) ? 1u : 0u;
+            p.text_tma = text_tensor_map(hm[0], d_texts[j], t.k, p.c_full, 32) &&
+                         (!p.mat || (text_tensor_map(hm[1], ws + t.L.off[24], t.k, p.c_full, 32) &&
+                                     text_tensor_map(hm[2], ws + t.L.off[25], t.k, p.c_full, 32))) ? 1u : 0u;
             p.state_tma = p.text_tma;
             p.tmaps = reinterpret_cast<const CUtensorMap *>(w + b->maps_off) + 3 * (size_t)t.slot;
         }
         std::memcpy(b->pinned + (size_t)t.slot * sizeof(Params), &p, sizeof(Params));
         outs[j].n_cols = t.len + 1;
     }
+    for (size_t j = 0; j < b->groups.size(); ++j) {          // the lane-walk groups' descriptors
+        const re_batch::Group &g = b->groups[j];
+        if (!g.walk) continue;
+        WalkGroup d{};
+        d.t = g.h->dev;
+        d.texts = reinterpret_cast<const Params *>(w + g.params_off);
+        d.chunk_base = reinterpret_cast<const uint64_t *>(w + g.cbase_off);
+        d.rtile_base = reinterpret_cast<const uint64_t *>(w + g.rbase_off);
+        d.mtile_base = reinterpret_cast<const uint64_t *>(w + g.mbase_off);
+        d.queue = reinterpret_cast<uint32_t *>(w + b->queue_off) + j * kQueues;
+        d.chunks = g.chunks; d.tiles = g.n_reach; d.mtiles = g.n_merge;
+        d.nt = (uint32_t)g.members.size();
+        d.per = g.per; d.logr = g.logr;
+        d.kind = g.kind; d.col_bytes = g.cb;
+        std::memcpy(b->pinned + b->wgroups_off + j * sizeof(WalkGroup), &d, sizeof(d));
+    }
+    b->wb.groups = reinterpret_cast<const WalkGroup *>(w + b->wgroups_off);
+    b->wb.heads = reinterpret_cast<const WalkSpan *>(w + b->heads_off);
+    b->wb.walk = reinterpret_cast<const WalkSpan *>(w + b->walk_off);
+    b->wb.gather = reinterpret_cast<const WalkSpan *>(w + b->gather_off);
+    b->wb.texts = reinterpret_cast<const Params *>(w);
+    b->wb.nt = count;
     cudaStream_t s = (cudaStream_t)stream;
     CUDA_TRY(cudaMemcpyAsync(w, b->pinned, b->desc_bytes, cudaMemcpyHostToDevice, s), "batch descriptor upload");
     CUDA_TRY(cudaEventRecord(b->uploaded, s), "batch event");

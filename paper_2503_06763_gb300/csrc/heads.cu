@@ -54,7 +54,24 @@ __device__ __forceinline__ void merge_runs(uint32_t (&s)[kRuns], uint32_t (&k)[k
     for (int j = 0; j < kRuns; ++j) { s[j] = ns[j]; k[j] = nk[j]; }
 }
 
+// The chunks of a kernel: one text's, or those of every text of a batch group.
+struct OneText {
+    const Params &p;
+    __device__ const DevTables &tables() const { return p.t; }
+    __device__ const Params &text(uint32_t) const { return p; }
+    __device__ uint32_t index(uint64_t first, uint32_t q, uint32_t) const { return (uint32_t)(first + q); }
+    __device__ uint32_t find(uint64_t) const { return 0; }
+};
+struct GroupTexts {
+    const WalkGroup &g;
+    __device__ const DevTables &tables() const { return g.t; }
+    __device__ const Params &text(uint32_t ti) const { return g.texts[ti]; }
+    __device__ uint32_t index(uint64_t first, uint32_t q, uint32_t ti) const { return (uint32_t)(first + q - __ldg(g.chunk_base + ti)); }
+    __device__ uint32_t find(uint64_t chunk) const { return text_of(g.chunk_base, g.nt, chunk); }
+};
+
 struct HeadShared {
+    uint32_t ti[kHeadChunks];                // the text of each chunk of the round
     uint8_t text[kHeadChunks * kHeadStride];
     uint32_t s[kRuns][kHeadChunks], k[kRuns][kHeadChunks], cnt[kHeadChunks], col[kHeadChunks];
     uint16_t wide[kHeadChunks];              // chunks of this round with more than kRuns slots: slots << 8 | chunk
@@ -65,8 +82,8 @@ struct HeadShared {
 template <bool FWD> struct HeadChunk {
     uint64_t base;
     uint32_t i, len, win;                    // window: bytes [win, win + kHeadWindow) of the chunk, inside it
-    __device__ HeadChunk(const Params &p, uint64_t first, uint32_t q) {
-        i = (uint32_t)(first + q);
+    __device__ HeadChunk(const Params &p, uint32_t chunk) {
+        i = chunk;
         base = (uint64_t)i * p.k;
         len = chunk_len(p, i);
         win = FWD || len <= kHeadWindow - 15 ? 0u : (len - (kHeadWindow - 15)) & ~15u;
@@ -87,15 +104,20 @@ __device__ __forceinline__ void head_word(const LaneTab &T, uint32_t w, uint32_t
 }
 
 // A round of a block: chunks first .. first + cnt - 1 (cnt <= per).
-template <bool FWD>
-__device__ void head_round(const Params &p, const LaneTab &T, HeadShared &S, uint64_t first, uint32_t cnt) {
-    const DevTables &t = p.t;
+template <bool FWD, typename Src>
+__device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint64_t first, uint32_t cnt) {
+    const DevTables &t = src.tables();
     const uint32_t ms = FWD ? t.msf : t.msb;
     const uint32_t *starts = FWD ? t.fSlotStart : t.bSlotStart;
     if (threadIdx.x == 0) S.nwide = 0;
+    if (threadIdx.x < cnt) S.ti[threadIdx.x] = src.find(first + threadIdx.x);
+    __syncthreads();
+    auto text_at = [&](uint32_t q) -> const Params & { return src.text(S.ti[q]); };
+    auto chunk_at = [&](uint32_t q) { return HeadChunk<FWD>(text_at(q), src.index(first, q, S.ti[q])); };
     // text windows, 16 bytes a thread
     for (uint32_t q = threadIdx.x; q < cnt * (kHeadWindow / 16); q += blockDim.x) {
-        const HeadChunk<FWD> c(p, first, q / (kHeadWindow / 16));
+        const Params &p = text_at(q / (kHeadWindow / 16));
+        const HeadChunk<FWD> c = chunk_at(q / (kHeadWindow / 16));
         const uint32_t at = 16 * (q % (kHeadWindow / 16));
         if (c.win + at < c.len) {
             const uint4 v = load16(p.x, p.n, c.base + c.win + at);
@@ -108,7 +130,8 @@ __device__ void head_round(const Params &p, const LaneTab &T, HeadShared &S, uin
     bool exact = false;
     if (threadIdx.x < cnt) {
         const uint32_t q = threadIdx.x;
-        const HeadChunk<FWD> c(p, first, q);
+        const Params &p = text_at(q);
+        const HeadChunk<FWD> c = chunk_at(q);
         exact = FWD ? (c.i == 0 && !(p.shard & SHARD_PREV)) : (c.i == p.c - 1 && !(p.shard & SHARD_NEXT));
         uint32_t m = 0;
         if (!exact) {
@@ -131,7 +154,8 @@ __device__ void head_round(const Params &p, const LaneTab &T, HeadShared &S, uin
     // chunks with more slots than a lane holds: a warp each, a lane per slot
     for (uint32_t r = threadIdx.x >> 5; r < S.nwide; r += blockDim.x / 32) {
         const uint32_t q = S.wide[r] & 0xFFu, m = S.wide[r] >> 8;
-        const HeadChunk<FWD> ch(p, first, q);
+        const Params &p = text_at(q);
+        const HeadChunk<FWD> ch = chunk_at(q);
         uint32_t v = lane < m ? __ldg(starts + (size_t)S.pr[q] * ms + lane) : 0u, c = FWD ? 1u : ch.len - 1;
         for (;;) {
             // to a multiple of four bytes, or the chunk's end
@@ -164,7 +188,8 @@ __device__ void head_round(const Params &p, const LaneTab &T, HeadShared &S, uin
     if (threadIdx.x < ((cnt + 31) & ~31u)) {
         const uint32_t q = threadIdx.x;
         const bool valid = q < cnt;
-        const HeadChunk<FWD> ch(p, first, valid ? q : 0);
+        const Params &p = text_at(valid ? q : 0);
+        const HeadChunk<FWD> ch = chunk_at(valid ? q : 0);
         const uint32_t nU = (ch.len + kUnit - 1) / kUnit;
         uint32_t s[kRuns], k[kRuns], n = 0, c = 0, conv = FWD ? 0 : nU, kind = 0;
         bool open = false, all = false;                       // all: every slot's end state is written already
@@ -258,19 +283,52 @@ __global__ void __launch_bounds__(kHeadThreads) heads_kernel(const __grid_consta
     stage_classes(p.t, cls);
     stage_lane_table<0>(backward ? p.t.bc8 : p.t.fc8, (backward ? p.t.nb : p.t.nf) * cw, sm);
     const uint64_t blk = pairs ? blockIdx.x >> 1 : blockIdx.x, nblk = pairs ? gridDim.x >> 1 : gridDim.x;
+    const OneText src{p};
     for (uint64_t first = blk * per; first < p.c; first += nblk * per) {   // head_round's first barrier: the tables are staged
         const uint32_t cnt = (uint32_t)min((uint64_t)per, p.c - first);
-        if (backward) head_round<false>(p, T, S, first, cnt);
-        else head_round<true>(p, T, S, first, cnt);
+        if (backward) head_round<false>(src, T, S, first, cnt);
+        else head_round<true>(src, T, S, first, cnt);
+    }
+}
+
+// Every lane-walk group of a batch: a block takes rounds of one group's chunks.
+__global__ void __launch_bounds__(kHeadThreads) heads_batch_kernel(const __grid_constant__ WalkBatch b) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ __align__(128) uint8_t cls[256];
+    __shared__ HeadShared S;
+    const bool pairs = !b.recognize, backward = pairs && (blockIdx.x & 1);
+    const WalkSpan w = b.heads[pairs ? blockIdx.x >> 1 : blockIdx.x];
+    const WalkGroup &g = b.groups[w.group];
+    const uint32_t cw = class_words(g.t);
+    const LaneTab T{smem_u32(sm), cls, cw * 4};
+    stage_classes(g.t, cls);
+    stage_lane_table<0>(backward ? g.t.bc8 : g.t.fc8, (backward ? g.t.nb : g.t.nf) * cw, sm);
+    const GroupTexts src{g};
+    for (uint64_t first = (uint64_t)w.idx * g.per; first < g.chunks; first += (uint64_t)w.cnt * g.per) {
+        const uint32_t cnt = (uint32_t)min((uint64_t)g.per, g.chunks - first);
+        if (backward) head_round<false>(src, T, S, first, cnt);
+        else head_round<true>(src, T, S, first, cnt);
     }
 }
 
 }  // namespace
 
+size_t heads_smem(const DevTables &t) { return (size_t)std::max(t.nf, t.nb) * class_words(t) * 4; }
+int heads_blocks_per_sm(size_t smem) {
+    static uint64_t attr_done = 0;
+    allow_smem(heads_batch_kernel, &attr_done);
+    int per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, heads_batch_kernel, kHeadThreads, smem);
+    return std::max(per_sm, 1);
+}
+void launch_heads_batch(const WalkBatch &b, cudaStream_t s) {
+    if (b.n_heads) heads_batch_kernel<<<b.n_heads * (b.recognize ? 1 : 2), kHeadThreads, b.heads_smem, s>>>(b);
+}
+
 // Chunks per block and round: kHeadChunks, fewer while that leaves the device
 // short of blocks (a warp takes about 1 us per chunk with many slots).
 void launch_heads(const Params &p, cudaStream_t s, int sm_count) {
-    const size_t smem = (size_t)std::max(p.t.nf, p.t.nb) * class_words(p.t) * 4;
+    const size_t smem = heads_smem(p.t);
     static uint64_t attr_done = 0;
     allow_smem(heads_kernel, &attr_done);
     int per_sm = 1;

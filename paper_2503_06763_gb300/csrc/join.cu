@@ -564,6 +564,40 @@ __global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_c
     if (blockIdx.x == 0 && threadIdx.x == 0) status_of(p);
 }
 
+// The same for every text of a batch's lane-walk groups, a block per text.
+// Chunks whose runs never met are evaluated in chains (a text of a batch has
+// few chunks).
+__global__ void join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    const Params &p = b.texts[blockIdx.x];
+    if (!p.rvar) return;                                      // a group of the other kernels
+    if (p.n == 0) {
+        if (threadIdx.x == 0) empty_text(p);
+        return;
+    }
+    if (p.w.scan[kScanGeneral]) {
+        for (uint32_t i = threadIdx.x; i < p.c; i += blockDim.x) chain_at(p, i);
+        __threadfence();
+        const uint32_t cw = class_words(p.t), nsf = p.t.nfd + 1, nsb = p.t.nbd + 1;
+        stage_classes(p.t, sm);
+        stage_lane_table<0>(p.t.fc8, nsf * cw, sm + 256);
+        stage_lane_table<0>(p.t.bc8, nsb * cw, sm + 256 + nsf * cw * 4);
+        __syncthreads();
+        const LaneTab F{smem_u32(sm + 256), sm, cw * 4}, B{smem_u32(sm + 256 + nsf * cw * 4), sm, cw * 4};
+        for (uint32_t i = threadIdx.x; i < p.c; i += blockDim.x) {
+            if (b.recognize) {
+                join_walk_fix<true, false>(p, F, nsf, i);
+            } else {
+                join_walk_fix<true, true>(p, F, nsf, i);
+                join_walk_fix<false, true>(p, B, nsb, i);
+            }
+        }
+        __threadfence();
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) status_of(p);
+}
+
 // ------------------------------------------------------------------ batch
 // The same steps over every chunk of every text of a group: thread j takes
 // flat chunk j (its text by binary search on the chunk prefix sums).
@@ -597,6 +631,7 @@ __global__ void batch_init_kernel(const Params *texts, uint32_t nt, uint32_t *qu
     if (j < nt && texts[j].n) {
         int32_t *f = texts[j].w.flags;
         for (uint32_t q = 0; q < FLAG_COUNT; ++q) f[q] = q < 2 ? (int32_t)texts[j].c : 0;
+        if (texts[j].rvar) texts[j].w.scan[kScanGeneral] = 0;
     }
 }
 
@@ -645,8 +680,17 @@ void launch_batch_init(const Params *texts, uint32_t nt, uint32_t *queues, uint3
     batch_init_kernel<<<(n + kBlockThreads - 1) / kBlockThreads, kBlockThreads, 0, s>>>(texts, nt, queues, nq);
 }
 
+size_t join_walk_smem(const DevTables &t) { return 256 + (size_t)(t.nfd + t.nbd + 2) * class_words(t) * 4; }
+
+void launch_join_walk_batch(const WalkBatch &b, cudaStream_t s) {
+    if (!b.nt) return;
+    static uint64_t attr_done = 0;
+    allow_smem(join_walk_batch_kernel, &attr_done);
+    join_walk_batch_kernel<<<b.nt, 128, b.join_smem, s>>>(b);
+}
+
 bool launch_join_walk(const Params &p, cudaStream_t s, int sm_count) {
-    const size_t smem = 256 + (size_t)(p.t.nfd + p.t.nbd + 2) * class_words(p.t) * 4;
+    const size_t smem = join_walk_smem(p.t);
     static uint64_t attr_done = 0;
     allow_smem(join_walk_kernel, &attr_done);
     return launch_coop(join_walk_kernel, smem, p.c, s, sm_count, p);

@@ -75,8 +75,7 @@ struct Params {
     uint32_t mat;                   // reach writes every position's state once its runs have met; the
                                     // fix-up fills the positions before; build & merge is a gather
     uint32_t state_tma;             // reach stores its state rows through TMA (mat)
-    uint32_t rvar;                  // reach shape (RE_PARSE_REACH): 1 byte tables, one direction per
-                                    // block; 2 / 3 warp pairs, 3 / 2 stages; 4 one lane per chunk
+    uint32_t rvar;                  // reach shape (RE_PARSE_REACH): 1 the lane walk; 2 / 3 warp pairs, 3 / 2 stages; 4 one lane per chunk
     uint32_t rstages;               // TMA ring stages of the warp-pair and one-lane shapes
     uint32_t rall;                  // the walk writes every slot's end state (slice maps), no columns
     uint32_t shard;                 // a slice of a longer text: SHARD_PREV, its first chunk speculates from
@@ -118,6 +117,33 @@ struct BatchGroup {
     uint32_t *queue;                // [kQueues] work counters, zeroed before the group runs
     uint64_t chunks, n_reach, n_merge;
     uint32_t nt, recognize;
+};
+// Groups of one batch that take the lane walk: every phase is one launch over
+// all of them.  A block belongs to one group (its tables are staged once): the
+// spans say which, and its place among the group's blocks.
+struct WalkGroup {
+    DevTables t;
+    const Params *texts;            // [nt], longest chunks first
+    const uint64_t *chunk_base;     // [nt+1] chunks before each text
+    const uint64_t *rtile_base;     // [nt+1] 32-chunk tiles before each text
+    const uint64_t *mtile_base;     // [nt+1] 2048-column tiles before each text
+    uint32_t *queue;                // [2] tiles handed out, forward and backward; zeroed before the walk
+    uint64_t chunks, tiles, mtiles;
+    uint32_t nt, per;               // per: chunks of a heads round
+    uint32_t logr;                  // table copies of the walk (walk.cu)
+    uint32_t kind, col_bytes;
+};
+struct WalkSpan {
+    uint32_t group, idx, cnt;       // block idx of cnt (per direction in the heads and the walk)
+};
+struct WalkBatch {
+    const WalkGroup *groups;
+    const WalkSpan *heads, *walk, *gather;   // a span per block (heads, walk: per pair of blocks, unless recognizing)
+    uint32_t n_heads, n_walk, n_gather;
+    uint32_t recognize;
+    size_t heads_smem, walk_smem, join_smem, gather_smem;
+    const Params *texts;            // every text of the batch (those of other groups have rvar 0)
+    uint32_t nt;
 };
 enum Queue { Q_REACH = 0, Q_MERGE = 1, kQueues = 4 };
 
@@ -212,21 +238,10 @@ __device__ inline void empty_text(const Params &p) {
 //   TM_SMEM8:  one-byte tables in shared memory as u8 (at most 256 states per
 //              direction; the reach's choice for larger class alphabets, a
 //              quarter of the u32 footprint, so more blocks fit an SM);
-//   TM_BYTE8:  tables indexed by the text byte itself (not its class), u8,
-//              rows of kByteRow bytes (256 entries and 4 of padding, which
-//              puts equal bytes of different states in different banks); a
-//              reach block stages one direction's table (about 65 KB).
-//   TM_BYTE7:  the same with rows of the bytes below 128 only (kAsciiRow
-//              bytes: 128 entries and 4 of padding, so entry (s, b) sits in
-//              bank (s + b / 4) mod 32 as in TM_BYTE8); the walk first
-//              replaces every byte >= 128 by a byte below 128 of its class
-//              (DevTables::hirep), which every class holding one has.
 // Row s, column = byte class (or class pair c1*ncls + c2 for the left and
 // right byte of the pair).  A forward pair consumes c1 then c2, a backward
 // pair c2 then c1.
-enum { TM_GLOBAL = 0, TM_SMEM = 1, TM_PAIR = 2, TM_SMEM8 = 3, TM_BYTE8 = 4, TM_BYTE7 = 5 };
-constexpr uint32_t kByteRow = 260;
-constexpr uint32_t kAsciiRow = 132;
+enum { TM_GLOBAL = 0, TM_SMEM = 1, TM_PAIR = 2, TM_SMEM8 = 3 };
 
 struct Tabs {
     const uint8_t *cls;
@@ -236,15 +251,12 @@ struct Tabs {
     const uint32_t *f2, *b2;
     uint32_t ncls, nc2;
     uint32_t rowb, nf, magic;       // reach in pair mode: run-state encoding (see reach_impl.cuh)
-    const uint8_t *rep;             // TM_BYTE7: [128] representative of byte b + 128 (shared memory)
 };
 
 template <int TM>
 __device__ __forceinline__ uint32_t fnext(const Tabs &T, uint32_t s, uint32_t c) {
     if (TM == TM_SMEM) return T.f16[s * T.ncls + c];
     if (TM == TM_SMEM8) return T.f8[s * T.ncls + c];
-    if (TM == TM_BYTE8) return T.f8[s * kByteRow + c];          // c is the byte itself
-    if (TM == TM_BYTE7) return T.f8[s * kAsciiRow + c];         // c is the byte, folded below 128
     if (TM == TM_PAIR) return T.f2[s * T.nc2 + c * T.ncls] & 0xFFFFu;
     return __ldg(T.f32 + (size_t)s * T.ncls + c);
 }
@@ -252,8 +264,6 @@ template <int TM>
 __device__ __forceinline__ uint32_t bnext(const Tabs &T, uint32_t s, uint32_t c) {
     if (TM == TM_SMEM) return T.b16[s * T.ncls + c];
     if (TM == TM_SMEM8) return T.b8[s * T.ncls + c];
-    if (TM == TM_BYTE8) return T.b8[s * kByteRow + c];
-    if (TM == TM_BYTE7) return T.b8[s * kAsciiRow + c];
     if (TM == TM_PAIR) return T.b2[s * T.nc2 + c] & 0xFFFFu;
     return __ldg(T.b32 + (size_t)s * T.ncls + c);
 }
@@ -262,76 +272,9 @@ __device__ __forceinline__ uint32_t bpair(const Tabs &T, uint32_t s, uint32_t cp
 
 template <int TM>
 __device__ __forceinline__ uint32_t clsof(const Tabs &T, uint32_t b) {
-    if (TM == TM_BYTE8 || TM == TM_BYTE7) return b;             // the tables are indexed by the byte
     if (TM != TM_GLOBAL) return T.cls[b];
     return __ldg(T.cls + b);
 }
-// The byte class itself (slot selection), in every table mode.
-template <int TM>
-__device__ __forceinline__ uint32_t class_of(const Tabs &T, const DevTables &t, uint32_t b) {
-    if (TM == TM_BYTE8 || TM == TM_BYTE7) return __ldg(t.cls + b);
-    return clsof<TM>(T, b);
-}
-
-// TM_BYTE7: bytes >= 128 of a word replaced by their representatives below
-// 128 (one shared-memory lookup per such byte; none for ASCII text).
-__device__ __forceinline__ uint32_t fold_word(const uint8_t *rep, uint32_t w) {
-    for (uint32_t hi = w & 0x80808080u; hi; hi &= hi - 1) {
-        const uint32_t sh = (uint32_t)__ffs(hi) - 8;             // the byte's lowest bit
-        w = (w & ~(0xFFu << sh)) | ((uint32_t)rep[(w >> sh) & 0x7Fu] << sh);
-    }
-    return w;
-}
-__device__ __forceinline__ uint4 fold_high_bytes(const uint8_t *rep, uint4 x) {
-    if (((x.x | x.y | x.z | x.w) & 0x80808080u) == 0) return x;
-    return make_uint4(fold_word(rep, x.x), fold_word(rep, x.y), fold_word(rep, x.z), fold_word(rep, x.w));
-}
-
-// Stage the byte-indexed tables of the directions asked for (block-wide;
-// ends with __syncthreads).  Returns the end of the used area.
-__device__ inline uint8_t *stage_byte8(const DevTables &t, uint8_t *sm, Tabs &T, bool fwd, bool bwd,
-                                       bool ascii = false) {
-    T.ncls = t.ncls;
-    T.nc2 = t.ncls * t.ncls;
-    T.cls = t.cls;
-    T.f32 = t.fT;
-    T.b32 = t.bT;
-    T.f16 = T.b16 = nullptr;
-    T.f2 = T.b2 = nullptr;
-    T.f8 = T.b8 = nullptr;
-    uint8_t *at = sm;
-    for (int d = 0; d < 2; ++d) {
-        if (!(d == 0 ? fwd : bwd)) continue;
-        const uint8_t *src = d == 0 ? t.fbyte : t.bbyte;
-        const uint32_t n = d == 0 ? t.nf : t.nb;
-        uint32_t *dst = reinterpret_cast<uint32_t *>(at);
-        const uint32_t *src32 = reinterpret_cast<const uint32_t *>(src);
-        if (ascii) {   // row s: the 32 words of bytes 0..127, then one word of padding
-            for (uint32_t q = threadIdx.x; q < n * 32; q += blockDim.x)
-                dst[(q >> 5) * (kAsciiRow / 4) + (q & 31)] = __ldg(src32 + (q >> 5) * 64 + (q & 31));
-        } else {       // row s: 64 words of entries, then one word of padding
-            for (uint32_t q = threadIdx.x; q < n * 64; q += blockDim.x)
-                dst[(q >> 6) * (kByteRow / 4) + (q & 63)] = __ldg(src32 + q);
-        }
-        (d == 0 ? T.f8 : T.b8) = at;
-        at += (((size_t)n * (ascii ? kAsciiRow : kByteRow)) + 15) & ~(size_t)15;
-    }
-    T.rep = nullptr;
-    if (ascii) {
-        for (uint32_t q = threadIdx.x; q < 32; q += blockDim.x)
-            reinterpret_cast<uint32_t *>(at)[q] = __ldg(reinterpret_cast<const uint32_t *>(t.hirep) + q);
-        T.rep = at;
-        at += 128;
-    }
-    __syncthreads();
-    return at;
-}
-__host__ __device__ inline size_t byte8_smem_bytes(const DevTables &t, bool fwd, bool bwd, bool ascii = false) {
-    const size_t row = ascii ? kAsciiRow : kByteRow;
-    return (fwd ? (((size_t)t.nf * row) + 15) & ~(size_t)15 : 0) +
-           (bwd ? (((size_t)t.nb * row) + 15) & ~(size_t)15 : 0) + (ascii ? 128 : 0);
-}
-
 // Bytes of shared memory used by stage_tables.
 __host__ __device__ inline size_t tables_smem_bytes(const DevTables &t, int tm) {
     if (tm == TM_GLOBAL) return 0;
@@ -526,13 +469,17 @@ __host__ __device__ inline DevTables dfa_tables(const DevTables &t) {
 }
 bool launch_reach(const Params &p, const CUtensorMap &text_map, const StateMaps &smaps, cudaStream_t s, uint32_t ms,
                   int sm_count);
-// Batch group with per-position states: the byte-table reach over its tiles,
-// the fix-up of the chunk heads and the gather of the columns.
-bool launch_reach_batch_byte8(const BatchGroup &b, uint32_t ms, cudaStream_t s, int sm_count);
-void launch_fixup_mat_batch(const BatchGroup &b, cudaStream_t s, int sm_count);
-void launch_gather_batch(const BatchGroup &b, const Params &like, cudaStream_t s, int sm_count);
-// Warps per direction of the byte-table reach (shape 1) on this device.
-uint64_t reach_byte8_warps(const Params &p, uint32_t ms, int sm_count);
+// The lane walk over the groups of a batch: one launch per phase.  The *_plan
+// functions give what a group needs of each.
+void launch_heads_batch(const WalkBatch &b, cudaStream_t s);
+void launch_walk_batch(const WalkBatch &b, cudaStream_t s);
+void launch_join_walk_batch(const WalkBatch &b, cudaStream_t s);
+void launch_gather_batch(const WalkBatch &b, cudaStream_t s);
+size_t heads_smem(const DevTables &t);
+size_t join_walk_smem(const DevTables &t);
+int walk_copies(const DevTables &t, uint64_t tiles, uint64_t blocks);   // log2
+size_t walk_smem_bytes(const DevTables &t, int logr);
+int heads_blocks_per_sm(size_t smem);
 // The lane walk (heads.cu, walk.cu) and the join after it.
 void launch_heads(const Params &p, cudaStream_t s, int sm_count);
 void launch_walk(const Params &p, const CUtensorMap &text_map, const StateMaps &smaps, cudaStream_t s, int sm_count);

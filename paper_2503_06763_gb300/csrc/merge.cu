@@ -882,24 +882,6 @@ __global__ void __launch_bounds__(kFixupThreads) fixup_mat_kernel(const __grid_c
     }
 }
 
-// Batch: items are (chunk, direction) over every text of the group.
-template <int TM>
-__global__ void __launch_bounds__(kFixupThreads) fixup_mat_batch_kernel(const __grid_constant__ BatchGroup b) {
-    extern __shared__ __align__(16) uint8_t sm[];
-    Tabs T;
-    stage_tables<TM>(dfa_tables(b.t), sm, T);
-    const uint64_t items = 2 * b.chunks;
-    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < items;
-         j += (uint64_t)gridDim.x * blockDim.x) {
-        const bool fwd = j < b.chunks;
-        const uint64_t f = fwd ? j : j - b.chunks;
-        const uint32_t ti = text_of(b.chunk_base, b.nt, f);
-        const Params &p = b.texts[ti];
-        if (*p.status != RE_OK) continue;                       // rejected: the gather writes zeros
-        fixup_mat_item<TM>(p, T, (uint32_t)(f - __ldg(b.chunk_base + ti)), fwd);
-    }
-}
-
 // The gather's encoder over classic-DFA state pairs, staged in shared memory
 // (the caller synchronises): the DICT pair table as 16-byte vectors of the
 // compiled copy (entry by entry from the 32-bit table of all states, a division
@@ -928,33 +910,62 @@ __device__ Enc stage_gather_enc(const DevTables &t, uint8_t *sm) {
     return e;
 }
 
+// True when a byte of the words is at least n (1 .. 256): the carry of its low
+// seven bits against n's, and its top bit, three operations per word.
+struct ByteBound {
+    uint32_t add, n;
+    __device__ __forceinline__ explicit ByteBound(uint32_t bound) : add((0x80u - (bound & 0x7Fu)) * 0x01010101u), n(bound) {}
+    __device__ __forceinline__ bool any(const uint4 &v) const {
+        if (n > 255) return false;
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t hit = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t low = (w[q] & 0x7F7F7F7Fu) + add;
+            hit |= n > 127 ? w[q] & low : w[q] | low;
+        }
+        return (hit & 0x80808080u) != 0;
+    }
+};
+
 // 16 columns from r0 on: their forward states a and backward states b (one
-// byte each) -> encoded columns, one 16-byte store per CB.
+// byte each) -> encoded columns, one 16-byte store per CB.  The states of all
+// 16 are checked against the classic DFAs first, so the lookups need no checks
+// of their own.
 template <int E>
 __device__ __forceinline__ void gather_unit(const Params &p, const Enc &e, uint32_t nfs, uint32_t nbs, bool ok,
                                             bool &bad, uint64_t r0, const uint4 &a, const uint4 &b) {
     constexpr int CB = bytes_of(E);
     const uint32_t fw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
     uint32_t ow[CB * 4];                                        // 16 columns of CB bytes
+    const bool fits = ok && !ByteBound(nfs).any(a) && !ByteBound(nbs).any(b);
+    if (fits) {
 #pragma unroll
-    for (int k = 0; k < CB * 4; ++k) ow[k] = 0;
+        for (int k = 0; k < 16; k += 4) {
+            uint64_t v[4];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const uint32_t f = (fw[k >> 2] >> (8 * (k & 3))) & 0xFFu, g = (bw[k >> 2] >> (8 * (k & 3))) & 0xFFu;
-        uint64_t v = 0;
-        if (ok) {
-            if (f >= nfs || g >= nbs) bad = true;
-            else v = enc_col<TM_SMEM, E>(e, f, g, bad);
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t f = __byte_perm(fw[k >> 2], 0u, 0x4440u | (uint32_t)u), g = __byte_perm(bw[k >> 2], 0u, 0x4440u | (uint32_t)u);
+                v[u] = enc_col<TM_SMEM, E>(e, f, g, bad);
+            }
+            if constexpr (CB == 8) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) { ow[2 * (k + u)] = (uint32_t)v[u]; ow[2 * (k + u) + 1] = (uint32_t)(v[u] >> 32); }
+            } else if constexpr (CB == 4) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) ow[k + u] = (uint32_t)v[u];
+            } else if constexpr (CB == 2) {
+                ow[k / 2] = __byte_perm((uint32_t)v[0], (uint32_t)v[1], 0x5410u);
+                ow[k / 2 + 1] = __byte_perm((uint32_t)v[2], (uint32_t)v[3], 0x5410u);
+            } else {
+                ow[k / 4] = __byte_perm(__byte_perm((uint32_t)v[0], (uint32_t)v[1], 0x0040u),
+                                        __byte_perm((uint32_t)v[2], (uint32_t)v[3], 0x0040u), 0x5410u);
+            }
         }
-        if constexpr (CB == 8) {
-            ow[2 * k] = (uint32_t)v;
-            ow[2 * k + 1] = (uint32_t)(v >> 32);
-        } else if constexpr (CB == 4) {
-            ow[k] = (uint32_t)v;
-        } else {
-            constexpr uint32_t m = (1u << (8 * CB)) - 1;
-            ow[(k * CB) >> 2] |= ((uint32_t)v & m) << (8 * ((k * CB) & 3));
-        }
+    } else {                                                    // rejected, or a state that no accepted text has
+        if (ok) bad = true;
+#pragma unroll
+        for (int k = 0; k < CB * 4; ++k) ow[k] = 0;
     }
     uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(p.out) + r0 * CB);
 #pragma unroll
@@ -1032,34 +1043,63 @@ __global__ void __launch_bounds__(kBlockThreads) merge_gather_kernel(const __gri
     if (bad) atomicExch(p.status, RE_E_INTERNAL);
 }
 
-// Batch: a warp per merge tile (2048 columns of one text of the group).
+// Every lane-walk group of a batch: a block takes tiles of 2048 columns of one
+// group's texts, a warp each, with four 16-byte loads per lane in flight.
 template <int E>
-__global__ void __launch_bounds__(kBlockThreads) gather_batch_kernel(const __grid_constant__ BatchGroup b) {
-    extern __shared__ __align__(16) uint8_t sm[];
-    const uint32_t nfs = b.t.nfd + 1, nbs = b.t.nbd + 1;
-    const Enc e = stage_gather_enc<E>(b.t, sm);
+__device__ void gather_group(const WalkGroup &g, const WalkSpan &sp, uint8_t *sm) {
+    const uint32_t nfs = g.t.nfd + 1, nbs = g.t.nbd + 1;
+    const Enc e = stage_gather_enc<E>(g.t, sm);
     __syncthreads();
-    const uint32_t lane = threadIdx.x & 31;
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
-    for (uint64_t tile = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; tile < b.n_merge; tile += warps) {
-        const uint32_t ti = text_of(b.mtile_base, b.nt, tile);
-        const Params &p = b.texts[ti];
+    const uint32_t lane = threadIdx.x & 31, wpb = blockDim.x / 32;
+    for (uint64_t tile = (uint64_t)sp.idx * wpb + (threadIdx.x >> 5); tile < g.mtiles; tile += (uint64_t)sp.cnt * wpb) {
+        const uint32_t ti = text_of(g.mtile_base, g.nt, tile);
+        const Params &p = g.texts[ti];
         const bool ok = *p.status == RE_OK;
         bool bad = false;
-        const uint64_t c0 = (tile - __ldg(b.mtile_base + ti)) * 2048;
+        const uint64_t c0 = (tile - __ldg(g.mtile_base + ti)) * 2048;
         const uint64_t c1 = min(c0 + 2048, p.n + 1);
         const uint4 zero = make_uint4(0, 0, 0, 0);
-        for (uint64_t r0 = c0 + 16 * lane; r0 + 16 <= c1; r0 += 512) {
-            uint4 a = zero, bb = zero;
-            if (ok) {
-                a = __ldcs(reinterpret_cast<const uint4 *>(p.w.FS + r0));
-                bb = __ldcs(reinterpret_cast<const uint4 *>(p.w.BS + r0));
+        const uint8_t *fs = p.w.FS, *bs = p.w.BS;
+#pragma unroll 1
+        for (uint64_t h = c0; h < c1; h += 1024) {
+            uint4 a[2], b[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint64_t r0 = h + 512 * q + 16 * lane;
+                const bool on = ok && r0 + 16 <= c1;
+                a[q] = on ? __ldcs(reinterpret_cast<const uint4 *>(fs + r0)) : zero;
+                b[q] = on ? __ldcs(reinterpret_cast<const uint4 *>(bs + r0)) : zero;
             }
-            gather_unit<E>(p, e, nfs, nbs, ok, bad, r0, a, bb);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint64_t r0 = h + 512 * q + 16 * lane;
+                if (r0 + 16 <= c1) gather_unit<E>(p, e, nfs, nbs, ok, bad, r0, a[q], b[q]);
+            }
         }
         const uint64_t tail = c0 + ((c1 - c0) & ~(uint64_t)15);   // fewer than 16 columns left
         if (tail + lane < c1) gather_one_column<E>(p, e, nfs, nbs, ok, bad, tail + lane);
         if (bad) atomicExch(p.status, RE_E_INTERNAL);
+    }
+}
+
+__global__ void __launch_bounds__(kBlockThreads, 4) gather_batch_kernel(const __grid_constant__ WalkBatch b) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    const WalkSpan sp = b.gather[blockIdx.x];
+    const WalkGroup &g = b.groups[sp.group];
+    if (g.kind == RE_SLPF_PAIRS) {
+        if (g.col_bytes == 4) gather_group<ENC_P4>(g, sp, sm);
+        else gather_group<ENC_P8>(g, sp, sm);
+    } else if (g.kind == RE_SLPF_DICT) {
+        if (g.col_bytes == 1) gather_group<ENC_X1>(g, sp, sm);
+        else if (g.col_bytes == 2) gather_group<ENC_X2>(g, sp, sm);
+        else gather_group<ENC_X4>(g, sp, sm);
+    } else {
+        switch (g.col_bytes) {
+            case 1: gather_group<ENC_D1>(g, sp, sm); break;
+            case 2: gather_group<ENC_D2>(g, sp, sm); break;
+            case 4: gather_group<ENC_D4>(g, sp, sm); break;
+            default: gather_group<ENC_D8>(g, sp, sm); break;
+        }
     }
 }
 
@@ -1253,41 +1293,11 @@ void launch_merge(const Params &p, const CUtensorMap &map, cudaStream_t s, int s
 
 void launch_empty(const Params &p, cudaStream_t s) { empty_text_kernel<<<1, 1, 0, s>>>(p); }
 
-void launch_fixup_mat_batch(const BatchGroup &b, cudaStream_t s, int sm_count) {
-    if (b.recognize || !b.chunks) return;
-    const size_t smem = tables_smem_bytes(dfa_tables(b.t), TM_SMEM8);
+void launch_gather_batch(const WalkBatch &b, cudaStream_t s) {
+    if (!b.n_gather) return;
     static uint64_t attr_done = 0;
-    allow_smem(fixup_mat_batch_kernel<TM_SMEM8>, &attr_done);
-    const int blocks = grid_for(fixup_mat_batch_kernel<TM_SMEM8>, smem, 2 * b.chunks, sm_count, kFixupThreads);
-    fixup_mat_batch_kernel<TM_SMEM8><<<blocks, kFixupThreads, smem, s>>>(b);
-}
-
-template <int E>
-void gather_batch_one(const BatchGroup &b, const Params &like, cudaStream_t s, int sm_count) {
-    const size_t smem = gather_smem(like);
-    static uint64_t attr_done = 0;
-    allow_smem(gather_batch_kernel<E>, &attr_done);
-    const int blocks = grid_for(gather_batch_kernel<E>, smem, b.n_merge * 32, sm_count, kBlockThreads);
-    gather_batch_kernel<E><<<blocks, kBlockThreads, smem, s>>>(b);
-}
-
-void launch_gather_batch(const BatchGroup &b, const Params &like, cudaStream_t s, int sm_count) {
-    if (b.recognize || !b.n_merge) return;
-    if (like.kind == RE_SLPF_PAIRS) {
-        if (like.col_bytes == 4) gather_batch_one<ENC_P4>(b, like, s, sm_count);
-        else gather_batch_one<ENC_P8>(b, like, s, sm_count);
-    } else if (like.kind == RE_SLPF_DICT) {
-        if (like.col_bytes == 1) gather_batch_one<ENC_X1>(b, like, s, sm_count);
-        else if (like.col_bytes == 2) gather_batch_one<ENC_X2>(b, like, s, sm_count);
-        else gather_batch_one<ENC_X4>(b, like, s, sm_count);
-    } else {
-        switch (like.col_bytes) {
-            case 1: gather_batch_one<ENC_D1>(b, like, s, sm_count); break;
-            case 2: gather_batch_one<ENC_D2>(b, like, s, sm_count); break;
-            case 4: gather_batch_one<ENC_D4>(b, like, s, sm_count); break;
-            default: gather_batch_one<ENC_D8>(b, like, s, sm_count); break;
-        }
-    }
+    allow_smem(gather_batch_kernel, &attr_done);
+    gather_batch_kernel<<<b.n_gather, kBlockThreads, b.gather_smem, s>>>(b);
 }
 
 void launch_fixup_batch(const BatchGroup &b, uint32_t tmode, cudaStream_t s, int sm_count) {

@@ -875,18 +875,11 @@ re_status compile_pattern(const char *pattern, size_t len, const re_compile_opts
                 for (size_t q = 0; q < cb; ++q) C.ptc[(f * nbs + b) * cb + q] = (uint8_t)(v >> (8 * q));
             }
     }
-    // ---- byte-indexed one-byte tables (states fit a byte): the reach looks a
-    // transition up by the text byte itself, with no class lookup first.
-    C.fbyte.clear(); C.bbyte.clear();
+    // ---- class-indexed one-byte rows of whole words (states fit a byte): the
+    // lane walk's tables
     C.fc8.clear(); C.bc8.clear();
+    C.ascii_rows = false;
     if (C.nf <= 256 && C.nb <= 256) {
-        C.fbyte.resize((size_t)C.nf * 256);
-        C.bbyte.resize((size_t)C.nb * 256);
-        for (uint32_t st = 0; st < C.nf; ++st)
-            for (uint32_t b = 0; b < 256; ++b) C.fbyte[(size_t)st * 256 + b] = (uint8_t)C.fT[(size_t)st * ncls + C.cls[b]];
-        for (uint32_t st = 0; st < C.nb; ++st)
-            for (uint32_t b = 0; b < 256; ++b) C.bbyte[(size_t)st * 256 + b] = (uint8_t)C.bT[(size_t)st * ncls + C.cls[b]];
-        // class-indexed rows of whole words (the lane walk's tables)
         const size_t row = 4 * ((size_t)(ncls + 3) / 4);
         C.fc8.assign(C.nf * row, 0);
         C.bc8.assign(C.nb * row, 0);
@@ -894,21 +887,11 @@ re_status compile_pattern(const char *pattern, size_t len, const re_compile_opts
             for (uint32_t c = 0; c < ncls; ++c) C.fc8[st * row + c] = (uint8_t)C.fT[(size_t)st * ncls + c];
         for (uint32_t st = 0; st < C.nb; ++st)
             for (uint32_t c = 0; c < ncls; ++c) C.bc8[st * row + c] = (uint8_t)C.bT[(size_t)st * ncls + c];
-    }
-    // ---- bytes 128..255 folded onto bytes below 128 of the same class: when
-    // every class holding a byte >= 128 also holds one below, the byte-indexed
-    // rows need only their first 128 entries (half the shared memory, so a
-    // reach block holds more warps), and a byte >= 128 is replaced by the
-    // smallest byte of its class before the lookup.
-    C.hirep.clear();
-    if (!C.fbyte.empty()) {
-        int rep[256];
-        for (int &r : rep) r = -1;
-        for (int b = 127; b >= 0; --b) rep[C.cls[b]] = b;
-        C.hirep.resize(128);
-        for (int b = 128; b < 256; ++b) {
-            if (rep[C.cls[b]] < 0) { C.hirep.clear(); break; }
-            C.hirep[b - 128] = (uint8_t)rep[C.cls[b]];
+        // every class holding a byte >= 128 also holds one below (re_info)
+        C.ascii_rows = true;
+        for (int b = 128; b < 256 && C.ascii_rows; ++b) {
+            C.ascii_rows = false;
+            for (int q = 0; q < 128 && !C.ascii_rows; ++q) C.ascii_rows = C.cls[q] == C.cls[b];
         }
     }
     C.fHash = build_device_hash(C.fBits, C.nf, W, C.fHashMask);

@@ -56,10 +56,7 @@ struct DevTables {
     const uint8_t *ptc;          // [nfd+1][nbd+1] the same over classic-DFA pairs, 1, 2 or 4 bytes an entry as
                                  // the DICT columns (0xFF.. for the others); null without a dictionary
     const uint32_t *f2, *b2;     // [n][ncls^2] two-byte tables (mid | end << 16), or null
-    const uint8_t *fbyte, *bbyte;  // [n][256] next state by byte (not class), u8; null unless n <= 256
     const uint8_t *fc8, *bc8;    // [n][4 * ceil(ncls / 4)] next state by class, u8; null unless n <= 256
-    const uint8_t *hirep;        // [128] byte b + 128 -> a byte below 128 of its class; null unless
-                                 // every class holding a byte >= 128 holds one below (and fbyte is set)
     uint32_t fHashMask, bHashMask;
     uint32_t ncls, W, ell;
     uint32_t nf, nb, nfd, nbd;   // states incl. empty row 0; nfd/nbd = classic DFA states
@@ -78,9 +75,8 @@ struct Compiled {
     uint32_t nf = 0, nb = 0, nfd = 0, nbd = 0, msf = 0, msb = 0;
     std::vector<uint32_t> fT, bT;             // [n][ncls]
     std::vector<uint32_t> f2, b2;             // [n][ncls^2] two-byte tables (empty when too large)
-    std::vector<uint8_t> fbyte, bbyte;        // [n][256] next state by byte (empty unless n <= 256)
     std::vector<uint8_t> fc8, bc8;            // [n][4 * ceil(ncls / 4)] next state by class (empty unless n <= 256)
-    std::vector<uint8_t> hirep;               // [128] representative below 128 of byte b + 128 (or empty)
+    bool ascii_rows = false;                  // every class holding a byte >= 128 holds one below (n <= 256)
     std::vector<uint64_t> fBits, bBits;       // [n][W]
     std::vector<uint32_t> fHash, bHash;
     uint32_t fHashMask = 0, bHashMask = 0;

@@ -139,14 +139,10 @@ __device__ __forceinline__ void walk_block(const Params &p, const Tabs &T, const
     const uint32_t swz = ((threadIdx.x & 31) >> 1) & 3;
 #pragma unroll 1
     for (int q = 0; q < 4; ++q) {
-        uint4 fx = FW ? *reinterpret_cast<const uint4 *>(frow + (((uint32_t)q ^ swz) << 4))
+        const uint4 fx = FW ? *reinterpret_cast<const uint4 *>(frow + (((uint32_t)q ^ swz) << 4))
                       : make_uint4(0, 0, 0, 0);
-        uint4 bx = bwd ? *reinterpret_cast<const uint4 *>(brow + (((uint32_t)(3 - q) ^ swz) << 4))
+        const uint4 bx = bwd ? *reinterpret_cast<const uint4 *>(brow + (((uint32_t)(3 - q) ^ swz) << 4))
                        : make_uint4(0, 0, 0, 0);
-        if (TM == TM_BYTE7) {                         // rows hold bytes below 128 only
-            if (FW) fx = fold_high_bytes(T.rep, fx);
-            if (bwd) bx = fold_high_bytes(T.rep, bx);
-        }
         if (TM == TM_PAIR && !EDGE) {                 // two bytes per table lookup (run states are row offsets)
             extern __shared__ __align__(16) uint8_t sm[];
             const uint32_t fw[4] = {fx.x, fx.y, fx.z, fx.w}, bw[4] = {bx.x, bx.y, bx.z, bx.w};
@@ -196,8 +192,7 @@ struct Ring {
     uint8_t *tiles;       // [nst][2][kTileBytes], 1024-byte aligned
     uint32_t bars;        // shared address of nst mbarriers
     uint32_t phase;       // bit s: parity of the next completion of stage s
-    uint32_t nst = kStages;   // stages (kStages; 2 in the one-direction-per-block kernel)
-    uint32_t nout = 2;        // MAT: state tiles per warp (2; 1 in the one-direction-per-block kernel)
+    uint32_t nst = kStages;   // stages
     uint32_t obuf = 0;        // MAT: the state tile the next block fills; it alternates across the
                               // warp's chunk tiles too, so the wait before a fill (at most one store
                               // group still reading) always concerns the other tile
@@ -310,7 +305,6 @@ __device__ __forceinline__ void walk_local(const Tabs &T, const uint8_t *row, ui
     for (int u = 0; u < hi - lo; ++u) {
         const int t = FWD ? lo + u : hi - 1 - u;
         uint32_t b = row[((((uint32_t)t >> 4) ^ swz) << 4) | ((uint32_t)t & 15)];
-        if (TM == TM_BYTE7 && b >= 128) b = T.rep[b - 128];
         const uint32_t c = clsof<T1>(T, b);
         for (uint32_t j = 0; j < m; ++j) s[j] = FWD ? fnext<T1>(T, s[j], c) : bnext<T1>(T, s[j], c);
         compact_local(s, mk, m);
@@ -394,7 +388,7 @@ __device__ bool reach_chunk(const Params &p, const Tabs &T, uint32_t i, const CU
     } else if (i == 0 && !(p.shard & SHARD_PREV)) {
         mf = 1; sf[0] = enc_f<TM>(T, t.fI); kf[0] = 1; tstart = 0;      // J_0 = I (a slice: its entry state)
     } else {
-        const uint32_t pr = class_of<TM>(T, t, __ldg(p.x + base - 1)) * t.ncls + class_of<TM>(T, t, __ldg(p.x + base));
+        const uint32_t pr = clsof<TM>(T, __ldg(p.x + base - 1)) * t.ncls + clsof<TM>(T, __ldg(p.x + base));
         mf = __ldg(t.fSlotCount + pr);
         if (WIDE && mf > (uint32_t)MS) {
             big = true;
@@ -411,8 +405,8 @@ __device__ bool reach_chunk(const Params &p, const Tabs &T, uint32_t i, const CU
         if (i == p.c - 1 && !(p.shard & SHARD_NEXT)) {
             mb = 1; sb[0] = enc_b<TM>(T, t.bF); kb[0] = 1; tlast = (int)len - 1;   // Ĵ_{c+1} = F (or the slice's)
         } else {
-            const uint32_t pr = class_of<TM>(T, t, __ldg(p.x + base + len - 1)) * t.ncls +
-                                class_of<TM>(T, t, __ldg(p.x + base + len));
+            const uint32_t pr = clsof<TM>(T, __ldg(p.x + base + len - 1)) * t.ncls +
+                                clsof<TM>(T, __ldg(p.x + base + len));
             mb = __ldg(t.bSlotCount + pr);
             if (WIDE && mb > (uint32_t)MS) {
                 big = true;
@@ -483,10 +477,7 @@ __device__ bool reach_chunk(const Params &p, const Tabs &T, uint32_t i, const CU
         const uint32_t wm = max(wmf, wmb);
         uint8_t *orow = MAT ? otile + ring.obuf * kTileBytes + lane * 64 : nullptr;
         if (MAT && tma) {                                     // the store that last used this tile has read it
-            if (lane == 0) {
-                if (ring.nout == 1) bulk_wait_read_all();
-                else bulk_wait_read_1();
-            }
+            if (lane == 0) bulk_wait_read_1();
             __syncwarp();
         }
         if (edge) {
@@ -529,7 +520,7 @@ __device__ bool reach_chunk(const Params &p, const Tabs &T, uint32_t i, const CU
                     }
                 }
             }
-            if (ring.nout == 2) ring.obuf ^= 1u;
+            ring.obuf ^= 1u;
         }
         if (WIDE && big) {                                    // this lane's runs past the register arrays
             if (FW) walk_local<TM, true>(T, frow, xs, xk, mx, f_lo, f_hi);
@@ -669,227 +660,6 @@ __global__ void __launch_bounds__(kSplitThreads, (SPLIT && MS <= 8) ? 3 : 1)
         }
     }
     if (MAT && lane == 0) bulk_wait_all();                    // state rows written before the grid ends
-}
-
-// One parse with byte-indexed tables (TM_BYTE8, or TM_BYTE7 when the bytes
-// >= 128 fold onto ASCII bytes of their class): every warp of a block walks
-// the same direction, so a block stages one direction's table (about 65 KB
-// for 251 states; half that with ASCII rows) instead of both.  Even blocks
-// walk 32-chunk tiles forward, odd blocks backward (every block forward in
-// recognizer mode); 2-stage TMA rings, and (MAT) one state tile per warp,
-// whose store has read it before the next block's states go in.  A warp's
-// lookups wait on shared-memory latency, so the block takes as many warps as
-// the shared memory left by its table holds (24 with full rows; up to 32
-// with ASCII rows, whose kernel is compiled for 1024 threads).  Tiles are
-// dealt round-robin over the blocks of a direction (tile t to block t mod
-// B), so a text of few tiles still spreads over every SM.
-constexpr uint32_t kDirThreads = 768;
-constexpr uint32_t kDirThreadsAscii = 1024;
-constexpr uint32_t kDirStages = 2;
-constexpr uint32_t kDirOut = 1;             // MAT state tiles per warp
-// Shared memory after the table: [1024-byte pad][text tiles, kDirStages per
-// warp][state tiles, kDirOut per warp][mbarriers, kDirStages per warp]; the
-// tiles are 1024-byte multiples, so one pad aligns them all.
-template <bool ASC> constexpr uint32_t dir_threads_max() { return ASC ? kDirThreadsAscii : kDirThreads; }
-
-inline size_t dir_table_smem(const DevTables &t, bool asc) {
-    return std::max(byte8_smem_bytes(t, true, false, asc), byte8_smem_bytes(t, false, true, asc));
-}
-inline size_t dir_warp_smem(bool mat) { return (kDirStages + (mat ? kDirOut : 0)) * kTileBytes + kDirStages * 8; }
-// Warps per block: as many as the shared memory holds, at most the kernel's bound.
-inline uint32_t dir_wpb(const DevTables &t, bool mat, bool asc) {
-    const size_t cap = asc ? kDirThreadsAscii / 32 : kDirThreads / 32;
-    const size_t avail = 227 * 1024 - dir_table_smem(t, asc) - 1024;
-    return (uint32_t)std::max<size_t>(1, std::min(cap, avail / dir_warp_smem(mat)));
-}
-inline size_t reach_dir_smem(const DevTables &t, bool mat, bool asc) {
-    return dir_table_smem(t, asc) + 1024 + dir_wpb(t, mat, asc) * dir_warp_smem(mat);
-}
-
-template <int MS, bool WIDE, bool MAT, bool ASC>
-__global__ void __launch_bounds__(dir_threads_max<ASC>(), 1)
-    reach_dir_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap map,
-                     const __grid_constant__ StateMaps smaps) {
-    constexpr int TM = ASC ? TM_BYTE7 : TM_BYTE8;
-    extern __shared__ __align__(16) uint8_t sm[];
-    const bool pairs = !p.recognize;
-    const bool backward_block = pairs && (blockIdx.x & 1);
-    Tabs T;
-    uint8_t *rest = stage_byte8(p.t, sm, T, !backward_block, backward_block, ASC);
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x / 32;
-    uint8_t *otile = nullptr;
-    Ring ring{};
-    ring.nst = kDirStages;
-    ring.nout = kDirOut;
-    {
-        const uint32_t a = smem_u32(rest);
-        uint8_t *aligned = rest + ((1024 - (a & 1023)) & 1023);
-        const uint32_t outs = MAT ? kDirOut : 0;
-        ring.tiles = aligned + warp * (kDirStages * kTileBytes);
-        ring.bars = smem_u32(aligned + wpb * (kDirStages + outs) * kTileBytes) + warp * kDirStages * 8;
-        ring.phase = 0;
-        if (MAT) otile = aligned + wpb * kDirStages * kTileBytes + warp * kDirOut * kTileBytes;
-        if (p.text_tma && lane == 0) {
-            for (uint32_t st = 0; st < kDirStages; ++st) mbar_init(ring.bars + 8 * st, 1);
-            mbar_init_fence();
-        }
-        __syncwarp();
-    }
-    pdl_wait();
-    pdl_trigger();
-    const uint64_t gblk = pairs ? blockIdx.x >> 1 : blockIdx.x, nblk = pairs ? gridDim.x >> 1 : gridDim.x;
-    for (uint64_t t = (uint64_t)warp * nblk + gblk; t * 32 < p.c; t += nblk * wpb) {
-        const uint32_t i = (uint32_t)(t * 32) + lane;
-        const bool tma = p.text_tma && t * 32 + 32 <= p.c_full;
-        if (i >= p.c) continue;                               // lanes past the text (plain path only)
-        const bool ok = backward_block
-                            ? reach_chunk<TM, MS, DIR_B, WIDE, MAT>(p, T, i, &map, ring, tma, &smaps.b, otile)
-                            : reach_chunk<TM, MS, DIR_F, WIDE, MAT>(p, T, i, &map, ring, tma, &smaps.f, otile);
-        if (!ok) {
-            atomicExch(p.status, RE_E_INTERNAL);
-            atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
-            for (uint32_t st = 0; st < kDirStages; ++st) {   // drain: bounded wait on every stage
-                bool done = false;
-                for (uint32_t it = 0; it < kWaitLimit && !done; ++it)
-                    done = mbar_try_wait(ring.bars + 8 * st, (ring.phase >> st) & 1u);
-            }
-            if (MAT && lane == 0) bulk_wait_all();
-            return;
-        }
-    }
-    if (MAT && lane == 0) bulk_wait_all();
-}
-
-// Blocks per direction: every resident block slot, split between the
-// directions, but no more blocks per direction than tiles (tiles go
-// round-robin over blocks).
-template <int MS, bool WIDE, bool MAT, bool ASC>
-uint64_t dir_blocks(const Params &p, int sm_count) {
-    const size_t smem = reach_dir_smem(p.t, MAT, ASC);
-    static uint64_t attr_done = 0;
-    allow_smem(reach_dir_kernel<MS, WIDE, MAT, ASC>, &attr_done, 227 * 1024);
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reach_dir_kernel<MS, WIDE, MAT, ASC>,
-                                                  dir_wpb(p.t, MAT, ASC) * 32, smem);
-    const uint64_t tiles = ((uint64_t)p.c + 31) / 32;
-    const uint64_t dirs = p.recognize ? 1 : 2;
-    const uint64_t slots = (uint64_t)std::max(per_sm, 1) * sm_count;
-    return std::max<uint64_t>(1, std::min<uint64_t>(tiles, slots / dirs));
-}
-
-template <int MS, bool WIDE, bool MAT, bool ASC>
-void launch_dir(const Params &p, const CUtensorMap &map, const StateMaps &smaps, cudaStream_t s, int sm_count) {
-    const size_t smem = reach_dir_smem(p.t, MAT, ASC);
-    const uint64_t dirs = p.recognize ? 1 : 2;
-    const uint64_t per_dir = dir_blocks<MS, WIDE, MAT, ASC>(p, sm_count);
-    const uint64_t blocks = per_dir * dirs;                    // even: one block of each pair per direction
-    launch_dependent(reach_dir_kernel<MS, WIDE, MAT, ASC>, (uint32_t)std::max<uint64_t>(blocks, 1),
-                     dir_wpb(p.t, MAT, ASC) * 32, smem, s, p, map, smaps);
-}
-
-// A batch group (one RE) with byte-indexed tables and per-position states:
-// the single-text kernel's shape (blocks alternate directions, one table per
-// block) over the 32-chunk tiles of every text of the group, dealt
-// round-robin over the blocks; full tiles of texts with tensor maps move by
-// TMA, the rest by plain loads and stores.
-template <int MS, bool WIDE, bool ASC>
-__global__ void __launch_bounds__(dir_threads_max<ASC>(), 1) reach_dir_batch_kernel(const __grid_constant__ BatchGroup b) {
-    constexpr int TM = ASC ? TM_BYTE7 : TM_BYTE8;
-    extern __shared__ __align__(16) uint8_t sm[];
-    const bool backward_block = blockIdx.x & 1;
-    Tabs T;
-    uint8_t *rest = stage_byte8(b.t, sm, T, !backward_block, backward_block, ASC);
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x / 32;
-    Ring ring{};
-    ring.nst = kDirStages;
-    ring.nout = kDirOut;
-    const uint32_t a = smem_u32(rest);
-    uint8_t *aligned = rest + ((1024 - (a & 1023)) & 1023);
-    ring.tiles = aligned + warp * (kDirStages * kTileBytes);
-    ring.bars = smem_u32(aligned + wpb * (kDirStages + kDirOut) * kTileBytes) + warp * kDirStages * 8;
-    ring.phase = 0;
-    uint8_t *otile = aligned + wpb * kDirStages * kTileBytes + warp * kDirOut * kTileBytes;
-    if (lane == 0) {
-        for (uint32_t st = 0; st < kDirStages; ++st) mbar_init(ring.bars + 8 * st, 1);
-        mbar_init_fence();
-    }
-    __syncwarp();
-    const uint64_t gblk = blockIdx.x >> 1, nblk = gridDim.x >> 1;
-    for (uint64_t t = (uint64_t)warp * nblk + gblk; t < b.n_reach; t += nblk * wpb) {
-        const uint32_t ti = text_of(b.rtile_base, b.nt, t);
-        const Params &p = b.texts[ti];
-        const uint64_t tile = t - __ldg(b.rtile_base + ti);
-        const uint32_t i = (uint32_t)(tile * 32) + lane;
-        // full tiles of a text with tensor maps go through TMA (text in, state rows out)
-        const bool tma = p.text_tma && p.state_tma && tile * 32 + 32 <= p.c_full;
-        if (tma && lane == 0) {
-            tensormap_acquire(p.tmaps);
-            tensormap_acquire(p.tmaps + (backward_block ? 2 : 1));
-        }
-        if (tma) __syncwarp();
-        if (i >= p.c) continue;                               // lanes past the text's last chunk (plain tiles only)
-        const bool ok = backward_block
-                            ? reach_chunk<TM, MS, DIR_B, WIDE, true>(p, T, i, p.tmaps, ring, tma, p.tmaps + 2, otile)
-                            : reach_chunk<TM, MS, DIR_F, WIDE, true>(p, T, i, p.tmaps, ring, tma, p.tmaps + 1, otile);
-        if (!ok) {
-            atomicExch(p.status, RE_E_INTERNAL);
-            for (uint32_t st = 0; st < kDirStages; ++st) {   // drain: bounded wait on every stage
-                bool done = false;
-                for (uint32_t it = 0; it < kWaitLimit && !done; ++it)
-                    done = mbar_try_wait(ring.bars + 8 * st, (ring.phase >> st) & 1u);
-            }
-            if (lane == 0) bulk_wait_all();
-            return;
-        }
-    }
-    if (lane == 0) bulk_wait_all();
-}
-
-template <int MS, bool WIDE, bool ASC>
-void launch_dir_batch_one(const BatchGroup &b, cudaStream_t s, int sm_count) {
-    const size_t smem = reach_dir_smem(b.t, true, ASC);
-    const uint32_t threads = dir_wpb(b.t, true, ASC) * 32;
-    static uint64_t attr_done = 0;
-    allow_smem(reach_dir_batch_kernel<MS, WIDE, ASC>, &attr_done, 227 * 1024);
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reach_dir_batch_kernel<MS, WIDE, ASC>, threads, smem);
-    const uint64_t slots = (uint64_t)std::max(per_sm, 1) * sm_count;
-    const uint64_t per_dir = std::max<uint64_t>(1, std::min<uint64_t>(b.n_reach, slots / 2));
-    reach_dir_batch_kernel<MS, WIDE, ASC><<<(uint32_t)(per_dir * 2), threads, smem, s>>>(b);
-}
-
-template <bool ASC>
-bool launch_dir_batch(const BatchGroup &b, uint32_t ms, cudaStream_t s, int sm_count) {
-    if (ms <= 2) launch_dir_batch_one<2, false, ASC>(b, s, sm_count);
-    else if (ms <= 4) launch_dir_batch_one<4, false, ASC>(b, s, sm_count);
-    else if (ms <= 8) launch_dir_batch_one<8, false, ASC>(b, s, sm_count);
-    else if (ms <= 32) launch_dir_batch_one<4, true, ASC>(b, s, sm_count);
-    else return false;
-    return true;
-}
-
-// Warps per direction the one-direction-per-block reach runs at most (every
-// resident block of a direction, dir_wpb warps each).
-template <bool MAT, bool ASC>
-uint64_t dir_warps(const Params &p, uint32_t ms, int sm_count) {
-    Params q = p;
-    q.c = 0xFFFFFFFFu;                                         // as many tiles as block slots
-    const uint64_t b = ms <= 2 ? dir_blocks<2, false, MAT, ASC>(q, sm_count)
-                     : ms <= 4 ? dir_blocks<4, false, MAT, ASC>(q, sm_count)
-                     : ms <= 8 ? dir_blocks<8, false, MAT, ASC>(q, sm_count)
-                               : dir_blocks<4, true, MAT, ASC>(q, sm_count);
-    return b * dir_wpb(p.t, MAT, ASC);
-}
-
-template <bool MAT, bool ASC>
-bool launch_dir_ms(const Params &p, const CUtensorMap &map, const StateMaps &smaps, cudaStream_t s, uint32_t ms,
-                   int sm_count) {
-    if (ms <= 2) launch_dir<2, false, MAT, ASC>(p, map, smaps, s, sm_count);
-    else if (ms <= 4) launch_dir<4, false, MAT, ASC>(p, map, smaps, s, sm_count);
-    else if (ms <= 8) launch_dir<8, false, MAT, ASC>(p, map, smaps, s, sm_count);
-    else if (ms <= 32) launch_dir<4, true, MAT, ASC>(p, map, smaps, s, sm_count);
-    else return false;
-    return true;
 }
 
 // Batch: warps take work items from the group's list (an atomic counter).  An

@@ -194,6 +194,53 @@ inline uint32_t walk_wpb(const DevTables &t) {               // warps a block's 
     return fixed >= kWalkSmemMax ? 0u : (uint32_t)std::min<size_t>(kWalkWarps, (kWalkSmemMax - fixed) / kWalkWarpSmem);
 }
 
+// A block's tables, tiles and barriers.
+struct WalkBlock {
+    LaneTab T;
+    WalkRing ring;
+    uint32_t ns;
+};
+template <int LOGR>
+__device__ __forceinline__ WalkBlock walk_setup(const DevTables &t, bool backward, uint32_t wpb, uint8_t *sm, uint8_t *cls) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cw = class_words(t);
+    WalkBlock w;
+    w.ns = (backward ? t.nbd : t.nfd) + 1;
+    uint8_t *tiles = sm + ((1024 - (smem_u32(sm) & 1023)) & 1023);
+    uint8_t *tab = tiles + wpb * 2 * kWalkTile;
+    w.ring = WalkRing{tiles + warp * 2 * kWalkTile, smem_u32(tab + lane_table_bytes<LOGR>(t)) + warp * 16, 0};
+    if (lane == 0 && warp < wpb) {
+        mbar_init(w.ring.bars, 1);
+        mbar_init(w.ring.bars + 8, 1);
+        mbar_init_fence();
+    }
+    w.T.cls = cls;
+    w.T.tab = smem_u32(tab) + (lane & ((1u << LOGR) - 1)) * 4;
+    w.T.rowb = (cw * 4) << LOGR;
+    stage_classes(t, cls);
+    stage_lane_table<LOGR>(backward ? t.bc8 : t.fc8, w.ns * cw, tab);
+    __syncthreads();
+    return w;
+}
+
+// One 32-chunk tile of a text; false: a lost TMA completion, after which the
+// loads in flight are given a bounded wait more.
+template <int LOGR, bool OUT>
+__device__ __forceinline__ bool walk_tile(const Params &p, WalkBlock &w, bool backward, uint64_t tile, const CUtensorMap *map,
+                                          const CUtensorMap *fmap, const CUtensorMap *bmap) {
+    const bool wide = (reinterpret_cast<uintptr_t>(p.x) & 31) == 0;
+    const bool ok = backward ? walk_chunk<LOGR, false, OUT>(p, w.T, w.ns, tile, wide, map, bmap, w.ring)
+                             : walk_chunk<LOGR, true, OUT>(p, w.T, w.ns, tile, wide, map, fmap, w.ring);
+    __syncwarp();
+    if (ok) return true;
+    atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
+    for (uint32_t st = 0; st < 2; ++st) {
+        bool done = false;
+        for (uint32_t it = 0; it < kWaitLimit && !done; ++it)
+            done = mbar_try_wait(w.ring.bars + 8 * st, (w.ring.phase >> st) & 1u);
+    }
+    return false;
+}
+
 template <int LOGR, bool OUT>
 __global__ void __launch_bounds__(kWalkWarps * 32, 1)
     walk_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap map,
@@ -201,42 +248,57 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1)
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ __align__(128) uint8_t cls[256];              // a fixed address: the lookups' offset is an immediate
     const bool pairs = !p.recognize, backward = pairs && (blockIdx.x & 1);
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x / 32;
-    const uint32_t cw = class_words(p.t), ns = (backward ? p.t.nbd : p.t.nfd) + 1;
-    uint8_t *tiles = sm + ((1024 - (smem_u32(sm) & 1023)) & 1023);
-    uint8_t *tab = tiles + wpb * 2 * kWalkTile;
-    WalkRing ring{tiles + warp * 2 * kWalkTile, smem_u32(tab + lane_table_bytes<LOGR>(p.t)) + warp * 16, 0};
-    if (lane == 0) {
-        mbar_init(ring.bars, 1);
-        mbar_init(ring.bars + 8, 1);
-        mbar_init_fence();
-    }
-    LaneTab T;
-    T.cls = cls;
-    T.tab = smem_u32(tab) + (lane & ((1u << LOGR) - 1)) * 4;
-    T.rowb = (cw * 4) << LOGR;
-    stage_classes(p.t, cls);
-    stage_lane_table<LOGR>(backward ? p.t.bc8 : p.t.fc8, ns * cw, tab);
-    __syncthreads();
+    const uint32_t warp = threadIdx.x >> 5, wpb = blockDim.x / 32;
+    WalkBlock w = walk_setup<LOGR>(p.t, backward, wpb, sm, cls);
     pdl_wait();
     pdl_trigger();
-    const bool wide = (reinterpret_cast<uintptr_t>(p.x) & 31) == 0;
     const uint64_t gblk = pairs ? blockIdx.x >> 1 : blockIdx.x, nblk = pairs ? gridDim.x >> 1 : gridDim.x;
-    for (uint64_t t = (uint64_t)warp * nblk + gblk; t * 32 < p.c; t += nblk * wpb) {
-        const bool ok = backward ? walk_chunk<LOGR, false, OUT>(p, T, ns, t, wide, &map, &smaps.b, ring)
-                                 : walk_chunk<LOGR, true, OUT>(p, T, ns, t, wide, &map, &smaps.f, ring);
-        __syncwarp();
-        if (!ok) {                                            // a bounded wait more for the loads in flight
-            atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
-            for (uint32_t st = 0; st < 2; ++st) {
-                bool done = false;
-                for (uint32_t it = 0; it < kWaitLimit && !done; ++it)
-                    done = mbar_try_wait(ring.bars + 8 * st, (ring.phase >> st) & 1u);
-            }
-            break;
-        }
-    }
+    for (uint64_t t = (uint64_t)warp * nblk + gblk; t * 32 < p.c; t += nblk * wpb)
+        if (!walk_tile<LOGR, OUT>(p, w, backward, t, &map, &smaps.f, &smaps.b)) break;
     if (OUT) bulk_wait_all();                                 // states written before the grid ends
+}
+
+// Every lane-walk group of a batch: a block takes tiles of one group's texts,
+// its warps from the group's queue of its direction (the tiles differ in
+// length and come longest first; dealt round-robin instead, 768 texts of 1 KiB
+// to 4 MiB took 0.52 ms; from the queue, and with whole tiles, 0.39 ms).
+template <int LOGR, bool OUT>
+__device__ void walk_group(const WalkBatch &b, const WalkGroup &g, const WalkSpan &sp, bool backward, uint8_t *sm, uint8_t *cls) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t fixed = 1024 + lane_table_bytes<LOGR>(g.t);  // warps this group's tables leave room for
+    const uint32_t wpb = min(blockDim.x / 32, (uint32_t)((b.walk_smem - fixed) / kWalkWarpSmem));
+    WalkBlock w = walk_setup<LOGR>(g.t, backward, wpb, sm, cls);
+    if (warp >= wpb) return;
+    for (;;) {
+        uint32_t t = 0;
+        if (lane == 0) t = atomicAdd(g.queue + (backward ? 1 : 0), 1u);
+        t = __shfl_sync(0xFFFFFFFFu, t, 0);
+        if (t >= g.tiles) break;
+        const uint32_t ti = text_of(g.rtile_base, g.nt, t);
+        const Params &p = g.texts[ti];
+        if (p.text_tma && lane == 0) {                        // maps in the descriptor area
+            tensormap_acquire(p.tmaps);
+            if (OUT) tensormap_acquire(p.tmaps + (backward ? 2 : 1));
+        }
+        __syncwarp();
+        if (!walk_tile<LOGR, OUT>(p, w, backward, t - __ldg(g.rtile_base + ti), p.tmaps, p.tmaps + 1, p.tmaps + 2)) break;
+    }
+    if (OUT) bulk_wait_all();
+}
+
+template <bool OUT>
+__global__ void __launch_bounds__(kWalkWarps * 32, 1) walk_batch_kernel(const __grid_constant__ WalkBatch b) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ __align__(128) uint8_t cls[256];
+    const bool pairs = !b.recognize, backward = pairs && (blockIdx.x & 1);
+    const WalkSpan sp = b.walk[pairs ? blockIdx.x >> 1 : blockIdx.x];
+    const WalkGroup &g = b.groups[sp.group];
+    switch (g.logr) {
+        case 5: walk_group<5, OUT>(b, g, sp, backward, sm, cls); break;
+        case 4: walk_group<4, OUT>(b, g, sp, backward, sm, cls); break;
+        case 2: walk_group<2, OUT>(b, g, sp, backward, sm, cls); break;
+        default: walk_group<0, OUT>(b, g, sp, backward, sm, cls); break;
+    }
 }
 
 // Table copies: as many of 32, 16 or 4 as leave room for kWalkMinWarps warps.
@@ -270,6 +332,25 @@ void walk_any(const Params &p, const CUtensorMap &map, const StateMaps &smaps, c
 }
 
 }  // namespace
+
+int walk_copies(const DevTables &t, uint64_t tiles, uint64_t blocks) { return walk_logr(t, tiles, blocks); }
+size_t walk_smem_bytes(const DevTables &t, int logr) {
+    const size_t tab = logr == 5 ? lane_table_bytes<5>(t) : logr == 4 ? lane_table_bytes<4>(t)
+                     : logr == 2 ? lane_table_bytes<2>(t) : lane_table_bytes<0>(t);
+    return std::min<size_t>(kWalkSmemMax - 256, 1024 + tab + kWalkWarps * kWalkWarpSmem);
+}
+void launch_walk_batch(const WalkBatch &b, cudaStream_t s) {
+    if (!b.n_walk) return;
+    const uint32_t blocks = b.n_walk * (b.recognize ? 1 : 2);
+    static uint64_t attr_out = 0, attr_rec = 0;
+    if (b.recognize) {
+        allow_smem(walk_batch_kernel<false>, &attr_rec, (int)kWalkSmemMax - 256);
+        walk_batch_kernel<false><<<blocks, kWalkWarps * 32, b.walk_smem, s>>>(b);
+    } else {
+        allow_smem(walk_batch_kernel<true>, &attr_out, (int)kWalkSmemMax - 256);
+        walk_batch_kernel<true><<<blocks, kWalkWarps * 32, b.walk_smem, s>>>(b);
+    }
+}
 
 void launch_walk(const Params &p, const CUtensorMap &map, const StateMaps &smaps, cudaStream_t s, int sm_count) {
     if (p.mat) walk_any<true>(p, map, smaps, s, sm_count);
