@@ -242,7 +242,7 @@ bool in_device_memory(const void *ptr) {
 // Shared memory the merge's encoder table takes when staged.
 size_t encoder_bytes(const DevTables &t, re_slpf_kind kind, uint32_t cb) {
     if (kind == RE_SLPF_PAIRS) return 0;
-    return kind == RE_SLPF_DICT ? (size_t)t.nf * t.nb * cb : (size_t)(t.nf + t.nb) * 8;
+    return kind == RE_SLPF_DICT ? 16 + dict_bytes(t, cb) : (size_t)(t.nf + t.nb) * 8;
 }
 
 uint32_t table_mode(const DevTables &t) {

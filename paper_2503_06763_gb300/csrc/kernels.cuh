@@ -290,6 +290,24 @@ __host__ __device__ inline size_t tables_smem_bytes(const DevTables &t, int tm) 
     return a;
 }
 
+// Entries 0 .. n - 1 of a table through this block's threads, kStageFlight of a
+// thread's loads in flight before their stores: staging waits on L2, and one
+// load at a time the 107,000 pairs of a 4109-state automaton were 105 of the
+// 120 us of build & merge of 64 KB of text (now 15).
+constexpr int kStageFlight = 8;
+template <typename Src, typename Put>
+__device__ __forceinline__ void stage_each(uint32_t n, Src src, Put put) {
+    for (uint32_t q = threadIdx.x; q < n; q += kStageFlight * blockDim.x) {
+        decltype(src(0u)) v[kStageFlight];
+#pragma unroll
+        for (int u = 0; u < kStageFlight; ++u)
+            if (q + u * blockDim.x < n) v[u] = src(q + u * blockDim.x);
+#pragma unroll
+        for (int u = 0; u < kStageFlight; ++u)
+            if (q + u * blockDim.x < n) put(q + u * blockDim.x, v[u]);
+    }
+}
+
 // Stage the byte-class map and the transition tables in shared memory
 // (block-wide; ends with __syncthreads).  Returns the end of the used area.
 template <int TM>
@@ -313,8 +331,8 @@ __device__ uint8_t *stage_tables(const DevTables &t, uint8_t *sm, Tabs &T) {
         const size_t fsz = (size_t)t.nf * t.ncls;
         uint16_t *b16 = reinterpret_cast<uint16_t *>(sm + 256 + ((fsz * 2 + 15) & ~(size_t)15));
         const size_t bsz = (size_t)t.nb * t.ncls;
-        for (size_t i = threadIdx.x; i < fsz; i += blockDim.x) f16[i] = (uint16_t)__ldg(t.fT + i);
-        for (size_t i = threadIdx.x; i < bsz; i += blockDim.x) b16[i] = (uint16_t)__ldg(t.bT + i);
+        stage_each((uint32_t)fsz, [&](uint32_t i) { return __ldg(t.fT + i); }, [&](uint32_t i, uint32_t v) { f16[i] = (uint16_t)v; });
+        stage_each((uint32_t)bsz, [&](uint32_t i) { return __ldg(t.bT + i); }, [&](uint32_t i, uint32_t v) { b16[i] = (uint16_t)v; });
         T.f16 = f16;
         T.b16 = b16;
         __syncthreads();
@@ -325,8 +343,8 @@ __device__ uint8_t *stage_tables(const DevTables &t, uint8_t *sm, Tabs &T) {
         const size_t fsz = (size_t)t.nf * t.ncls;
         uint8_t *b8 = f8 + ((fsz + 15) & ~(size_t)15);
         const size_t bsz = (size_t)t.nb * t.ncls;
-        for (size_t i = threadIdx.x; i < fsz; i += blockDim.x) f8[i] = (uint8_t)__ldg(t.fT + i);
-        for (size_t i = threadIdx.x; i < bsz; i += blockDim.x) b8[i] = (uint8_t)__ldg(t.bT + i);
+        stage_each((uint32_t)fsz, [&](uint32_t i) { return __ldg(t.fT + i); }, [&](uint32_t i, uint32_t v) { f8[i] = (uint8_t)v; });
+        stage_each((uint32_t)bsz, [&](uint32_t i) { return __ldg(t.bT + i); }, [&](uint32_t i, uint32_t v) { b8[i] = (uint8_t)v; });
         T.f8 = f8;
         T.b8 = b8;
         __syncthreads();
@@ -341,7 +359,7 @@ __device__ uint8_t *stage_tables(const DevTables &t, uint8_t *sm, Tabs &T) {
     if (contiguous && ((reinterpret_cast<uintptr_t>(t.f2) & 15) == 0)) {
         const uint4 *src = reinterpret_cast<const uint4 *>(t.f2);
         uint4 *dst = reinterpret_cast<uint4 *>(f2);
-        for (size_t i = threadIdx.x; i < nwords / 4; i += blockDim.x) dst[i] = __ldg(src + i);
+        stage_each((uint32_t)(nwords / 4), [&](uint32_t i) { return __ldg(src + i); }, [&](uint32_t i, uint4 v) { dst[i] = v; });
         for (size_t i = (nwords / 4) * 4 + threadIdx.x; i < nwords; i += blockDim.x) f2[i] = __ldg(t.f2 + i);
     } else {
         for (size_t i = threadIdx.x; i < (size_t)t.nf * nc2; i += blockDim.x) f2[i] = __ldg(t.f2 + i);
@@ -466,6 +484,10 @@ __host__ __device__ inline DevTables dfa_tables(const DevTables &t) {
     c.nf = t.nfd + 1;
     c.nb = t.nbd + 1;
     return c;
+}
+// The staged DICT pair table: classic-DFA pairs, whole 16-byte vectors.
+__host__ __device__ inline size_t dict_bytes(const DevTables &t, uint32_t cb) {
+    return ((size_t)(t.nfd + 1) * (t.nbd + 1) * cb + 15) & ~(size_t)15;
 }
 bool launch_reach(const Params &p, const CUtensorMap &text_map, const StateMaps &smaps, cudaStream_t s, uint32_t ms,
                   int sm_count);

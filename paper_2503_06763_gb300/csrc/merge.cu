@@ -366,7 +366,7 @@ struct Enc {
 template <int E>
 __device__ __forceinline__ uint32_t enc_lo(const Enc &e, uint32_t f, uint32_t b, bool &bad) {
     if (is_dict(E)) {
-        const uint32_t at = f * e.nb + b;                 // the pair table spans every state pair
+        const uint32_t at = f * e.nb + b;                 // staged: classic-DFA pairs; global: all pairs
         if (E == ENC_X1 && e.pt8) return e.pt8[at];
         return e.pt16 ? (uint32_t)e.pt16[at] : e.pt32[at];
     }
@@ -448,7 +448,7 @@ __device__ __forceinline__ void group_full(const Params &p, const Tabs &T, const
     auto cls_at = [&](int u) -> uint32_t { return (cw[u >> 2] >> (8 * (u & 3))) & 0xFFu; };
     uint32_t f = p.w.FC[g];
     uint32_t b = p.w.BC[g];                                    // B̂_64
-    if (f == kUnknown || b == kUnknown) { bad = true; f = 0; b = 0; }   // never index with the sentinel
+    if (f > p.t.nfd || b > p.t.nbd) { bad = true; f = 0; b = 0; }   // the sentinel, or no state of the text's own
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
         if (i > 0) f = fnext<TM>(T, f, cls_at(i - 1));        // B_i
@@ -507,7 +507,7 @@ __device__ __forceinline__ void group_full_pair(const Params &p, const Tabs &T, 
     auto cp_at = [&](int j) -> uint32_t { return (cpk[j >> 2] >> (8 * (j & 3))) & 0xFFu; };
     uint32_t f = p.w.FC[g];                                    // B_0
     uint32_t b = p.w.BC[g];                                    // B̂_64
-    if (f == kUnknown || b == kUnknown) { bad = true; f = 0; b = 0; }
+    if (f > p.t.nfd || b > p.t.nbd) { bad = true; f = 0; b = 0; }
     uint32_t sF[16], sB[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -573,7 +573,7 @@ __device__ __forceinline__ void group_full_reg(const Params &p, const Tabs &T, c
     auto cls_at = [&](int u) -> uint32_t { return (cw[u >> 2] >> (8 * (u & 3))) & 0xFFu; };
     uint32_t f = p.w.FC[g];                                    // B_0
     uint32_t b = p.w.BC[g];                                    // B̂_64
-    if (f == kUnknown || b == kUnknown || f > p.t.nfd || b > p.t.nbd) { bad = true; f = 0; b = 0; }
+    if (f > p.t.nfd || b > p.t.nbd) { bad = true; f = 0; b = 0; }
     uint32_t rF[16], rB[16];                                   // B_0..B_31; B̂_32..B̂_63 (two per word)
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
@@ -609,14 +609,14 @@ __device__ __forceinline__ void group_full_reg(const Params &p, const Tabs &T, c
 }
 
 // Last group (fewer than 64 columns or no byte after it): plain loops.
-template <int TM, int E, bool REG = false>
+template <int TM, int E>
 __device__ void group_tail(const Params &p, const Tabs &T, const Enc &e, uint64_t g, bool &bad) {
     const uint64_t pos = g * 64;
     const uint64_t nleft = p.n + 1 - pos;
     const uint32_t ncol = nleft < 64 ? (uint32_t)nleft : 64u;
     uint32_t F[64], B[64];
     uint32_t f = p.w.FC[g], b = p.w.BC[g];
-    if (f == kUnknown || b == kUnknown || (REG && (f > p.t.nfd || b > p.t.nbd))) { bad = true; f = 0; b = 0; }
+    if (f > p.t.nfd || b > p.t.nbd) { bad = true; f = 0; b = 0; }
     F[0] = f;
     for (uint32_t u = 1; u < ncol; ++u) F[u] = fnext<TM>(T, F[u - 1], clsof<TM>(T, __ldg(p.x + pos + u - 1)));
     if (pos + 64 <= p.n) b = bnext<TM>(T, b, clsof<TM>(T, __ldg(p.x + pos + 63)));
@@ -644,24 +644,15 @@ __device__ void merge_setup(const DevTables &t0, uint32_t enc_in_smem, uint8_t *
     if (is_pair(E)) {                                         // the state ids themselves: no encoder
     } else if (is_dict(E)) {
         if (enc_in_smem) {
-            const size_t cnt = (size_t)t.nf * t.nb;
-            const uint32_t nbs = t0.nb;                       // row stride of the device pair table
-            auto src = [&](size_t i) -> uint32_t {
-                return REG ? __ldg(t.pt + (i / t.nb) * nbs + i % t.nb) : __ldg(t.pt + i);
-            };
-            if (E == ENC_X1) {                                // indices below 255 (0xFF: never produced)
-                uint8_t *pt = rest;
-                for (size_t i = threadIdx.x; i < cnt; i += blockDim.x) pt[i] = (uint8_t)src(i);
-                e.pt8 = pt;
-            } else if (E == ENC_X2) {
-                uint16_t *pt = reinterpret_cast<uint16_t *>(rest);
-                for (size_t i = threadIdx.x; i < cnt; i += blockDim.x) pt[i] = (uint16_t)src(i);
-                e.pt16 = pt;
-            } else {
-                uint32_t *pt = reinterpret_cast<uint32_t *>(rest);
-                for (size_t i = threadIdx.x; i < cnt; i += blockDim.x) pt[i] = src(i);
-                e.pt32 = pt;
-            }
+            // the compiled copy over classic-DFA pairs, 16 bytes a load
+            const uint32_t cnt = (uint32_t)dict_bytes(t0, bytes_of(E)) / 16;
+            const uint4 *src = reinterpret_cast<const uint4 *>(t0.ptc);
+            uint4 *pt = reinterpret_cast<uint4 *>(base + ((rest - base + 15) & ~(size_t)15));
+            stage_each(cnt, [&](uint32_t i) { return __ldg(src + i); }, [&](uint32_t i, uint4 v) { pt[i] = v; });
+            e.nb = t0.nbd + 1;
+            if (E == ENC_X1) e.pt8 = reinterpret_cast<uint8_t *>(pt);
+            else if (E == ENC_X2) e.pt16 = reinterpret_cast<uint16_t *>(pt);
+            else e.pt32 = reinterpret_cast<uint32_t *>(pt);
         } else {
             e.pt32 = t.pt;
             e.nb = t0.nb;
@@ -669,8 +660,8 @@ __device__ void merge_setup(const DevTables &t0, uint32_t enc_in_smem, uint8_t *
     } else if (enc_in_smem) {                                 // DENSE: segment bitsets of the states
         uint64_t *fb = reinterpret_cast<uint64_t *>(rest);
         uint64_t *bb = fb + t.nf;
-        for (uint32_t i = threadIdx.x; i < t.nf; i += blockDim.x) fb[i] = __ldg(t.fBits + i);
-        for (uint32_t i = threadIdx.x; i < t.nb; i += blockDim.x) bb[i] = __ldg(t.bBits + i);
+        stage_each(t.nf, [&](uint32_t i) { return __ldg(t.fBits + i); }, [&](uint32_t i, uint64_t v) { fb[i] = v; });
+        stage_each(t.nb, [&](uint32_t i) { return __ldg(t.bBits + i); }, [&](uint32_t i, uint64_t v) { bb[i] = v; });
         e.fbits = fb; e.bbits = bb;
     } else {
         e.fbits = t.fBits; e.bbits = t.bBits;                 // too many states to stage
@@ -703,7 +694,7 @@ __device__ __forceinline__ void merge_group(const Params &p, const Tabs &T, cons
             group_full<TM, E, TMA, St>(p, T, e, g, bad, stage + threadIdx.x, stage + 32 * kBlockThreads + threadIdx.x,
                                        out);
     } else {
-        group_tail<TM, E, REG>(p, T, e, g, bad);
+        group_tail<TM, E>(p, T, e, g, bad);
     }
 }
 
@@ -893,7 +884,7 @@ __device__ Enc stage_gather_enc(const DevTables &t, uint8_t *sm) {
     Enc e{};
     e.nb = nbs;
     if constexpr (is_dict(E)) {
-        const uint32_t cnt = (uint32_t)(((size_t)nfs * nbs * bytes_of(E) + 15) / 16);
+        const uint32_t cnt = (uint32_t)dict_bytes(t, bytes_of(E)) / 16;
         const uint4 *src = reinterpret_cast<const uint4 *>(t.ptc);
 #pragma unroll 4
         for (uint32_t q = threadIdx.x; q < cnt; q += blockDim.x) reinterpret_cast<uint4 *>(sm)[q] = __ldg(src + q);
@@ -1214,7 +1205,7 @@ void fixup_one(const Params &p, cudaStream_t s, int sm_count) {
 size_t gather_smem(const Params &p) {
     const size_t nfs = p.t.nfd + 1, nbs = p.t.nbd + 1;
     if (p.kind == RE_SLPF_PAIRS) return 0;
-    return p.kind == RE_SLPF_DICT ? (nfs * nbs * p.col_bytes + 15) & ~(size_t)15 : (nfs + nbs) * 8;
+    return p.kind == RE_SLPF_DICT ? dict_bytes(p.t, p.col_bytes) : (nfs + nbs) * 8;
 }
 
 template <int TM>
@@ -1264,7 +1255,7 @@ size_t merge_extra_smem(const Params &p) {
     if (p.tmode != TM_PAIR && !p.merge_reg)
         a += (2 * 32 * kBlockThreads * (p.tmode == TM_GLOBAL ? 4 : 2) + 15) & ~(size_t)15;
     if (!p.enc_in_smem || p.kind == RE_SLPF_PAIRS) return a;
-    if (p.kind == RE_SLPF_DICT) return a + (size_t)t.nf * t.nb * p.col_bytes;
+    if (p.kind == RE_SLPF_DICT) return a + 16 + dict_bytes(p.t, p.col_bytes);
     return a + (size_t)(t.nf + t.nb) * 8;
 }
 

@@ -70,15 +70,16 @@ __device__ inline uint8_t *stage_reach_pair(const DevTables &t, uint8_t *sm, Tab
     }
     uint16_t *rows = reinterpret_cast<uint16_t *>(sm + kRows);
     const size_t nfw = (size_t)t.nf * nc2, nbw = (size_t)t.nb * nc2;
-    for (size_t i = threadIdx.x; i < nfw; i += blockDim.x) rows[i] = (uint16_t)((__ldg(t.f2 + i) >> 16) * rowb);
-    for (size_t i = threadIdx.x; i < nbw; i += blockDim.x)
-        rows[nfw + i] = (uint16_t)((t.nf + (__ldg(t.b2 + i) >> 16)) * rowb);
+    stage_each((uint32_t)nfw, [&](uint32_t i) { return __ldg(t.f2 + i); },
+               [&](uint32_t i, uint32_t v) { rows[i] = (uint16_t)((v >> 16) * rowb); });
+    stage_each((uint32_t)nbw, [&](uint32_t i) { return __ldg(t.b2 + i); },
+               [&](uint32_t i, uint32_t v) { rows[nfw + i] = (uint16_t)((t.nf + (v >> 16)) * rowb); });
     uint8_t *after = sm + kRows + (((nfw + nbw) * 2 + 15) & ~(size_t)15);
     uint16_t *f16 = reinterpret_cast<uint16_t *>(after);
     const size_t fsz = (size_t)t.nf * ncls, bsz = (size_t)t.nb * ncls;
     uint16_t *b16 = reinterpret_cast<uint16_t *>(after + ((fsz * 2 + 15) & ~(size_t)15));
-    for (size_t i = threadIdx.x; i < fsz; i += blockDim.x) f16[i] = (uint16_t)__ldg(t.fT + i);
-    for (size_t i = threadIdx.x; i < bsz; i += blockDim.x) b16[i] = (uint16_t)__ldg(t.bT + i);
+    stage_each((uint32_t)fsz, [&](uint32_t i) { return __ldg(t.fT + i); }, [&](uint32_t i, uint32_t v) { f16[i] = (uint16_t)v; });
+    stage_each((uint32_t)bsz, [&](uint32_t i) { return __ldg(t.bT + i); }, [&](uint32_t i, uint32_t v) { b16[i] = (uint16_t)v; });
     T.cls = sm + kCls;
     T.f16 = f16;
     T.b16 = b16;
