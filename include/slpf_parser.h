@@ -149,15 +149,18 @@ typedef struct {
  * end states and the same SLPF).  re_autotune chooses one per handle and
  * length bucket together with the chunk length; RE_PARSE_REACH(v) in
  * re_parse_opts.flags forces one (tests, measurements):
- *   1: tables indexed by the byte itself, one direction per block of 24
- *      warps (32 when every class with a byte >= 128 has one below, so the
- *      rows hold bytes 0..127 only), 2-stage TMA ring (automata of at most
- *      256 states per direction);
+ *   1: the lane walk: the speculative runs of every chunk's first bytes in a
+ *      kernel of their own, then one run per chunk and direction, a lane per
+ *      chunk, on through the next chunk's first bytes, over a copy of the
+ *      class-indexed tables for each lane (automata of at most 256 states per
+ *      direction);
  *   2: a warp per direction of each 32-chunk tile (two lanes per chunk),
  *      tables by byte class, 3-stage TMA ring;
  *   3: as 2 with a 2-stage ring;
  *   4: one lane per chunk walking both directions, 3-stage ring.
- * 0 (the default) is the tuned shape, else 1 where it applies, else 2.
+ * 0 (the default) is the tuned shape, else 1 where it applies and the
+ * two-byte tables of 2 do not fit shared memory or every text makes a chunk's
+ * runs meet within 64 letters, else 2.
  * Shapes 1 (and 2, 3 when the class alphabet is above 16) let the reach
  * store every position's state, so build & merge is a gather.              */
 #define RE_PARSE_REACH(v) ((uint32_t)(v) << 8)
@@ -199,8 +202,7 @@ typedef struct {
     uint32_t inf_ambiguous;   /* 1 when the RE is infinitely ambiguous (its SLPFs are samples) */
     uint32_t sample_limit;    /* the compile option's sample_limit */
     uint32_t ascii_rows;      /* 1 when every byte class holding a byte >= 128 also holds one
-                                 below 128: the byte-table reach then stages table rows of the
-                                 128 bytes below 128 only and folds the others onto them */
+                                 below 128 (automata of at most 256 states per direction) */
     uint32_t reach_shapes;    /* bit v set: reach shape v (RE_PARSE_REACH) runs for this automaton */
 } re_info;
 

@@ -5,6 +5,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <memory>
@@ -49,10 +50,22 @@ int sm_count_of(int device) {
     return c;
 }
 
-// The lane walk (RE_PARSE_REACH shape 1) is the built-in choice for automata of
-// at most 256 states whose two-byte tables do not fit shared memory.
 bool walks(const re_handle *h);
+bool scan_join(const re_handle *h);
 uint32_t table_mode(const DevTables &t);
+
+// The lane walk (RE_PARSE_REACH shape 1) is the built-in choice for automata of
+// at most 256 states: where their two-byte tables do not fit shared memory, and
+// where they do if every text makes a chunk's runs meet within kMeetMax letters
+// ((a|b|ab)* at 1 MiB 36 us against 59 for warp pairs, at 256 MiB 432 against
+// 470).  With small tables and runs that can stay apart, warp pairs are the
+// better ones: they take two bytes a lookup and the walk's join evaluates the
+// chunks whose runs never met ((aa)* at 64 MiB 475 us against 612 for the lane
+// walk, the genome RE at 256 MiB 594 against 791).
+constexpr uint32_t kMeetMax = 64;
+bool walk_first(const re_handle *h) {
+    return walks(h) && (table_mode(h->dev) == TM_SMEM || h->host.meet <= kMeetMax);
+}
 
 // n bytes over `target` chunks.
 uint32_t chunk_for(uint64_t n, uint64_t target) {
@@ -61,14 +74,33 @@ uint32_t chunk_for(uint64_t n, uint64_t target) {
     return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(k, 256), 1u << 20);
 }
 
+// One reach thread per chunk, about 2 resident warps per scheduler.  The layout
+// of this length is what a workspace must hold; where the rules below want one
+// that it does not hold as well, this length is taken.
+uint32_t plain_chunk(uint64_t n, int sms) { return chunk_for(n, (uint64_t)sms * 384); }
+
 // Chunk length k.  Lane walk: a lane per chunk, as many chunks as the device
-// walks at once in a direction.  Otherwise one reach thread per chunk, about 2
-// resident warps per scheduler, chunks long enough that speculative runs meet
-// early in them.
+// walks at once in a direction; but no more chunk heads than the device takes
+// at once (8 blocks of 64 per SM) while chunks are below 384 bytes, as a head
+// costs about as much as 100 bytes of walk (11 MiB of log text: 320 take 47 us
+// where 256 take 55; 12.5 MiB: 384 49, 256 64).
+// Warp pairs: the chunks of plain_chunk, or fewer where half of them or less
+// are better: a chunk's bytes are walked one after another, 24 ns each, and
+// each chunk costs the join about 4 ns when byte states make it a scan over all
+// chunks, and under 2 ns when it is not; the sum is least at k = sqrt(n / 8)
+// and about sqrt(n / 16).  Genome RE, 16 MiB: 320-byte chunks 254 us, 1472 159;
+// 1 MiB: 256 130, 384 120; 256 MiB: 5824 616, 4608 592.  (a|b)*a(a|b)^9, 16
+// MiB: 320 178, 1024 128.
 uint32_t choose_chunk(const re_handle *h, uint64_t n, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
     const bool rec = opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY);
-    return chunk_for(n, walks(h) && table_mode(h->dev) == TM_SMEM ? walk_lanes(h->dev, rec, sms) : (uint64_t)sms * 384);
+    if (walk_first(h)) {
+        const uint64_t heads = (uint64_t)sms * 8 * 64 / (rec ? 1 : 2);
+        return chunk_for(n, std::max(heads, std::min(n / 384, walk_lanes(h->dev, rec, sms))));
+    }
+    const uint64_t most = (uint64_t)sms * 384;
+    const uint64_t fewer = std::max<uint64_t>(1, (uint64_t)std::sqrt((scan_join(h) ? 8.0 : 16.0) * (double)n));
+    return chunk_for(n, fewer <= most / 2 ? fewer : most);
 }
 
 int length_bucket(uint64_t n) {
@@ -432,6 +464,8 @@ re_status re_workspace_size(const re_handle *h, uint64_t len, const re_parse_opt
     const uint32_t k = kt ? kt : choose_chunk(h, len, sm_count_of(h->device), opts);
     if (k % kSub || k == 0) { set_error("chunk_len must be a positive multiple of 64"); return RE_E_INVALID_ARG; }
     *bytes = layout_for(h, len, k, mat_for(h, opts)).total;
+    if (!kt && !(opts && opts->chunk_len))
+        *bytes = std::max(*bytes, (uint64_t)layout_for(h, len, plain_chunk(len, sm_count_of(h->device)), mat_for(h, opts)).total);
     return RE_OK;
 }
 
@@ -442,7 +476,7 @@ namespace slpf {
 // what re_parse falls back to when the workspace it is given cannot hold the
 // tuned layout.
 re_status workspace_rule_bytes(const re_handle *h, uint64_t len, const re_parse_opts *opts, uint64_t *bytes) {
-    const uint32_t k = choose_chunk(h, len, sm_count_of(h->device), opts);
+    const uint32_t k = opts && opts->chunk_len ? opts->chunk_len : plain_chunk(len, sm_count_of(h->device));
     if (k % kSub || k == 0) { set_error("chunk_len must be a positive multiple of 64"); return RE_E_INVALID_ARG; }
     *bytes = layout_for(h, len, k, mat_for(h, opts)).total;
     return RE_OK;
@@ -514,8 +548,11 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     if (dev_now != h->device) { set_error("current device differs from the handle's device"); return RE_E_INVALID_ARG; }
     const int sms = sm_count_of(h->device);
     uint32_t k = choose_chunk(h, len, sms, opts);
-    if (const uint32_t kt = tuned_chunk(h, len, opts)) {      // tuned length, if the workspace holds it
-        if (!len || layout_for(h, len, kt, mat_for(h, opts)).total <= workspace_bytes) k = kt;
+    if (len && !(opts && opts->chunk_len)) {
+        auto fits = [&](uint32_t v) { return layout_for(h, len, v, !map_mode && mat_for(h, opts)).total <= workspace_bytes; };
+        const uint32_t plain = plain_chunk(len, sms), kt = tuned_chunk(h, len, opts);
+        if (kt && fits(kt)) k = kt;                           // tuned length, if the workspace holds it
+        else if (!fits(plain) || !fits(k)) k = plain;
     }
     if (k % kSub || k == 0) { set_error("chunk_len must be a positive multiple of 64"); return RE_E_INVALID_ARG; }
     if (len / k >= 0xFFFFFFF0ull) { set_error("text too long for this chunk length"); return RE_E_INVALID_ARG; }
@@ -542,7 +579,7 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     p.tmode = table_mode(t);
     if (!shape) shape = tuned_shape(h, len, opts);            // chosen with the tuned chunk length
     if (!shape || !(shapes_of(h) >> shape & 1))
-        shape = (shapes_of(h) >> 1 & 1) && p.tmode == TM_SMEM ? 1u : 2u;
+        shape = walk_first(h) ? 1u : 2u;
     p.rvar = shape;
     p.rstages = shape == 3 ? 2u : 3u;
     const size_t tab = tables_smem_bytes(t, p.tmode);

@@ -345,6 +345,46 @@ class StateTable {
     std::vector<uint32_t> index_;
 };
 
+// Letters after which at most one of a chunk's speculative runs is alive and
+// apart from the others, whatever the text (kNever: some text keeps two apart
+// for ever): the longest path of state pairs from the pairs of one slot list,
+// none if the pairs reach a cycle.
+constexpr uint32_t kNever = 0xFFFFFFFFu;
+uint32_t meet_bound(const std::vector<uint32_t> &T, uint32_t n, uint32_t ncls,
+                    const std::vector<std::vector<uint32_t>> &slots) {
+    std::vector<uint32_t> len((size_t)n * n, kNever);         // of the pairs done (kNever: not met yet)
+    std::vector<uint8_t> open((size_t)n * n, 0);
+    struct Frame { uint32_t pair, cls, longest; };
+    std::vector<Frame> path;
+    auto pair_of = [n](uint32_t a, uint32_t b) { return a < b ? a * n + b : b * n + a; };
+    uint32_t bound = 0;
+    for (const auto &list : slots)
+        for (size_t i = 0; i < list.size(); ++i)
+            for (size_t j = i + 1; j < list.size(); ++j) {
+                const uint32_t first = pair_of(list[i], list[j]);
+                if (len[first] == kNever) { path.push_back({first, 0, 0}); open[first] = 1; }
+                while (!path.empty()) {
+                    Frame &f = path.back();
+                    if (f.cls == ncls) {
+                        const uint32_t l = len[f.pair] = f.longest + 1;
+                        open[f.pair] = 0;
+                        path.pop_back();
+                        if (!path.empty()) path.back().longest = std::max(path.back().longest, l);
+                        continue;
+                    }
+                    const uint32_t a = T[(size_t)(f.pair / n) * ncls + f.cls], b = T[(size_t)(f.pair % n) * ncls + f.cls];
+                    ++f.cls;
+                    if (a == b || !a || !b) continue;         // met, or one died
+                    const uint32_t q = pair_of(a, b);
+                    if (open[q]) return kNever;
+                    if (len[q] != kNever) f.longest = std::max(f.longest, len[q]);
+                    else { open[q] = 1; path.push_back({q, 0, 0}); }
+                }
+                bound = std::max(bound, len[first]);
+            }
+    return bound;
+}
+
 std::vector<uint32_t> build_device_hash(const std::vector<uint64_t> &bits, uint32_t n, uint32_t W,
                                         uint32_t &mask_out) {
     uint64_t cap = 16;
@@ -893,6 +933,16 @@ re_status compile_pattern(const char *pattern, size_t len, const re_compile_opts
             C.ascii_rows = false;
             for (int q = 0; q < 128 && !C.ascii_rows; ++q) C.ascii_rows = C.cls[q] == C.cls[b];
         }
+    }
+    C.meet = 0xFFFFFFFFu;
+    if (!C.fc8.empty() && !C.f2.empty()) {
+        auto starts = [&](const auto &slots) {
+            std::vector<std::vector<uint32_t>> v(slots.size());
+            for (size_t j = 0; j < slots.size(); ++j)
+                for (const auto &e : slots[j]) v[j].push_back(e.first);
+            return v;
+        };
+        C.meet = std::max(meet_bound(C.fT, C.nf, ncls, starts(fsl)), meet_bound(C.bT, C.nb, ncls, starts(bsl)));
     }
     C.fHash = build_device_hash(C.fBits, C.nf, W, C.fHashMask);
     C.bHash = build_device_hash(C.bBits, C.nb, W, C.bHashMask);

@@ -76,6 +76,7 @@ struct Compiled {
     std::vector<uint32_t> fT, bT;             // [n][ncls]
     std::vector<uint32_t> f2, b2;             // [n][ncls^2] two-byte tables (empty when too large)
     std::vector<uint8_t> fc8, bc8;            // [n][4 * ceil(ncls / 4)] next state by class (empty unless n <= 256)
+    uint32_t meet = 0xFFFFFFFFu;              // letters within which a chunk's runs always meet (two-byte tables, n <= 256)
     bool ascii_rows = false;                  // every class holding a byte >= 128 holds one below (n <= 256)
     std::vector<uint64_t> fBits, bBits;       // [n][W]
     std::vector<uint32_t> fHash, bHash;
