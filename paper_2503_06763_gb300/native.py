@@ -24,7 +24,7 @@ RE_COMPILE_DFA_STARTS = 2
 RE_COMPILE_DFA_STARTS_BWD = 4
 RE_PARSE_RECOGNIZE_ONLY = 1
 RE_PARSE_TEST_STALL_JOIN = 0x80000000     # tests of the join's bounded waits only
-REACH_SHAPES = {1: "byte tables, one direction per block, 2 stages", 2: "warp pairs, class tables, 3 stages",
+REACH_SHAPES = {1: "lane walk: heads, then a lane per chunk and direction", 2: "warp pairs, class tables, 3 stages",
                 3: "warp pairs, class tables, 2 stages", 4: "one lane per chunk, both directions, 3 stages"}
 
 
@@ -609,14 +609,17 @@ def slpf_dfa_encode(cols, text, interval: int = 4096):
         raise ValueError("one column per position 0..n")
     lib = load()
     size = ctypes.c_uint64()
-    st = lib.re_slpf_dfa_encode(cols.ctypes.data, cols.dtype.itemsize, x.ctypes.data if x.size else None, x.size,
-                                interval, None, 0, ctypes.byref(size))
-    if st not in (RE_OK, -8):
-        check(st)
-    out = np.zeros(size.value, dtype=np.uint8)
-    check(lib.re_slpf_dfa_encode(cols.ctypes.data, cols.dtype.itemsize, x.ctypes.data if x.size else None, x.size,
-                                 interval, out.ctypes.data, out.size, ctypes.byref(size)))
-    return out
+    # room that most archives fit in (its pages are touched only as far as the
+    # archive goes), so that the columns are encoded once; else the size reported
+    room = (1 << 20) + min(4 * x.size, 1 << 28)
+    while True:
+        out = np.empty(room, dtype=np.uint8)
+        st = lib.re_slpf_dfa_encode(cols.ctypes.data, cols.dtype.itemsize, x.ctypes.data if x.size else None, x.size,
+                                    interval, out.ctypes.data, out.size, ctypes.byref(size))
+        if st != -8 or size.value <= room:
+            check(st)
+            return out[:size.value].copy()
+        room = size.value
 
 
 def slpf_dfa_header(archive) -> dict:
