@@ -169,21 +169,26 @@ def cpu_baseline(text_host, pattern, sample_bytes):
 
 def lsu_roofline(phase_ms: dict, n: int, device: int, ncls: int, shape: int):
     """Reach against the shared-memory pipe, its real bound.  Shared-memory
-    lookups per text byte: 2 with byte-indexed tables (reach shape 1: one
-    transition per byte and direction); with class tables 3 for at most 16
-    byte classes (per direction and byte pair: two class lookups and one
-    two-byte table lookup), else 4 (per direction and byte: one class and one
-    transition lookup).  Peak: one 32-lane wavefront per SM and cycle at the
+    lookups per text byte: 3 with class tables for at most 16 byte classes
+    (per direction and byte pair: two class lookups and one two-byte table
+    lookup), else 4, as in the lane walk (reach shape 1; per direction and
+    byte: one class and one transition lookup).  Peak: one 32-lane wavefront per SM and cycle at the
     maximum SM clock (bank conflicts make a lookup cost more)."""
     import torch
     props = torch.cuda.get_device_properties(device)
     peak = props.multi_processor_count * 32 * 2.07e9 / 1e12
-    per_byte = 2 if shape == 1 else 3 if ncls <= 16 else 4
+    per_byte = 3 if shape != 1 and ncls <= 16 else 4
     achieved = per_byte * n / (phase_ms["reach"] / 1e3) / 1e12
     return {"kernel": "reach", "bound": "lsu", "lookups_per_byte": per_byte, "achieved": round(achieved, 3),
             "peak": round(peak, 3),
             "unit": "T lookups/s", "frac": round(achieved / peak, 4),
             "peak_source": "SM count x 32 lanes x 2070 MHz (one conflict-free wavefront per SM and cycle)"}
+
+
+def launches_per_parse(shape: int) -> int:
+    """Kernels of one parse: heads, walk, join and gather in the lane walk; else
+    flags, reach, three joins, fix-up, build & merge."""
+    return 4 if shape == 1 else 7
 
 
 # The sources of the kernels whose DRAM traffic profiles/traffic.json records
@@ -300,7 +305,7 @@ def measure_single(args, name, n, rank, world, local, dist, full=True):
                 for j, p in enumerate(PHASES)}
     dominant = max(phase_ms, key=phase_ms.get)
     shape = args.reach_shape if args.chunk_len else rx.tuned(n)[1]
-    if not shape:                       # the library's default: byte tables when they fit, else warp pairs
+    if not shape:                       # the library's default: the lane walk unless two-byte tables fit
         shape = 1 if rx.info["n_classes"] > 16 and rx.info["fwd_states"] < 256 and rx.info["bwd_states"] < 256 else 2
     # algorithmic bytes per launch: text read once, plus the SLPF written by build & merge
     alg = {"reach": n, "join": 0, "fixup": 0, "build_merge": n + (n + 1) * cb}
@@ -449,7 +454,7 @@ def main():
         "warmup": args.warmup, "ms_per_step": r["ms_per_step"], "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "u8", "data": "synthetic", "config": r["config"],
         "roofline": r["roofline"], "cpu_baseline": r.get("cpu_baseline"), "e2e": r.get("e2e"),
-        "recognizer": r.get("recognizer"), "gpu_launches": 7 * args.steps, "clocks": r["clocks"],
+        "recognizer": r.get("recognizer"), "gpu_launches": launches_per_parse(r["config"]["reach_shape"]) * args.steps, "clocks": r["clocks"],
     }
     if extra:
         line["dna"] = extra
@@ -580,7 +585,7 @@ def batch_mode(args, rank, world, local):
                    "segments": [r[2].ell for r in res], "encodings": sorted(set(kinds))},
         "graph_replay": {"value": gbs(ms_graph), "ms_per_step": round(ms_graph, 3)},
         "per_text_launches": {"value": gbs(ms_single), "ms_per_step": round(ms_single, 3),
-                              "launches_per_step": 7 * args.texts},
+                              "launches_per_step": launches_per_parse(1) * args.texts},
         "roofline": {"bound": "hbm", "achieved": round((total + out_bytes) / (ms_batch / 1e3) / 1e9, 1),
                      "peak": hbm, "peak_source": src, "unit": "GB/s",
                      "frac": round((total + out_bytes) / (ms_batch / 1e3) / 1e9 / hbm, 4)},
@@ -741,7 +746,7 @@ def matches_mode(args, rank, world, local):
 
 def latency_mode(args, rank, world, local):
     """One small text, (a|b|ab)* over 1 MiB of uniform a/b (seed 0): latency of
-    one parse with its 7 launches issued directly, and as a CUDA-graph
+    one parse with its launches issued directly, and as a CUDA-graph
     replay of the same re_parse call."""
     import numpy as np
     import torch

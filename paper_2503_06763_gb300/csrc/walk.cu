@@ -13,7 +13,7 @@
 // no tiles and no barriers, but costs a wavefront per lane and access, 0.27 ms
 // at 256 MiB of log text.
 //
-// Measured (heads and walk together, log text): 11 MiB 55 us, 256 MiB 0.27 ms,
+// Measured (heads and walk together, log text): 11 MiB 47 us, 256 MiB 0.27 ms,
 // 1 GiB 0.97 ms = 4.3 TB/s of text read and states written, where one kernel
 // of byte-indexed tables that held a chunk's runs in registers and local
 // memory took 140 us, 0.37 ms and 1.10 ms and left the chunk heads to another.
