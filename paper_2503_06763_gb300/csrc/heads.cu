@@ -158,8 +158,9 @@ __device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint
         const HeadChunk<FWD> ch = chunk_at(q);
         uint32_t v = lane < m ? __ldg(starts + (size_t)S.pr[q] * ms + lane) : 0u, c = FWD ? 1u : ch.len - 1;
         for (;;) {
-            // to a multiple of four bytes, or the chunk's end
-            const uint32_t to = FWD ? min((c + 4) & ~3u, ch.len) : (c - 1) & ~3u;
+            // to a multiple of four bytes, or the chunk's end; a chunk of one byte starts at its end
+            // (backward c is 0 then), its slots' states are its end states
+            const uint32_t to = FWD ? min((c + 4) & ~3u, ch.len) : (max(c, 1u) - 1) & ~3u;
             while (c != to) {
                 const uint32_t at = FWD ? c : c - 1, w = at - ch.win;
                 v = lane_step<0>(T, v, w < kHeadWindow ? S.text[q * kHeadStride + w] : __ldg(p.x + ch.base + at));
