@@ -32,6 +32,7 @@ constexpr uint32_t kDfaMagic = 0x46504C53u;   // "SLPF"
 constexpr uint32_t kDfaVersion = 2;
 constexpr uint32_t kNoEntry = 0xFFFFu;          // a table entry no (column, byte) pair filled
 constexpr uint32_t kMaxIds = 65535;            // ids fit u16 beside kNoEntry (tables of at most 32 MiB)
+constexpr uint32_t kDecodeTableThread = 200 * 1024;   // table bytes a thread-per-piece block stages at most
 constexpr uint32_t kMaxInterval = 65536;       // exception offsets within a piece fit u16
 
 size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }
@@ -425,18 +426,22 @@ __global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kern
     if (bad) atomicExch(a.status, RE_E_INTERNAL);
 }
 
+// The shared-memory limit of each kernel is raised once, to the most any archive
+// takes: a limit per call would be another thread's limit between its launch
+// and the call that set it.
 template <int CB, bool BYTE>
 cudaError_t launch_decode_warp(const DecodeArgs &a, cudaStream_t s, int sms) {
+    constexpr uint32_t warps = decode_warps<CB>(), warp_smem = tile_bytes<CB>() + kDecodeExc * 4;
     const uint32_t windows = (a.interval + kWindow - 1) / kWindow;
     const uint32_t table = std::min<uint32_t>(kDecodeTable, (uint32_t)(((size_t)a.n_ids * (260 + 4) * (BYTE ? 1 : 2) + 15) / 16 * 16));
-    const size_t smem = table + decode_warps<CB>() * (tile_bytes<CB>() + kDecodeExc * 4);
-    const cudaError_t e = cudaFuncSetAttribute(slpf_dfa_warp_kernel<CB, BYTE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    const size_t smem = table + warps * warp_smem;
+    static uint64_t attr_done = 0;
+    allow_smem(slpf_dfa_warp_kernel<CB, BYTE>, &attr_done, kDecodeTable + warps * warp_smem);
     int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slpf_dfa_warp_kernel<CB, BYTE>, decode_warps<CB>() * 32, smem);
-    const uint64_t want = (a.n_checkpoints * windows + decode_warps<CB>() - 1) / decode_warps<CB>();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slpf_dfa_warp_kernel<CB, BYTE>, warps * 32, smem);
+    const uint64_t want = (a.n_checkpoints * windows + warps - 1) / warps;
     const uint32_t blocks = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * std::max(per_sm, 1)));
-    slpf_dfa_warp_kernel<CB, BYTE><<<blocks, decode_warps<CB>() * 32, smem, s>>>(a, table, windows);
+    slpf_dfa_warp_kernel<CB, BYTE><<<blocks, warps * 32, smem, s>>>(a, table, windows);
     return cudaGetLastError();
 }
 
@@ -521,15 +526,10 @@ extern "C" re_status re_slpf_dfa_decode(const re_slpf_dfa_header *hdr, const voi
     a.out = d_cols;
     a.status = d_status;
     const size_t tab_bytes = (size_t)hdr->n_ids * 256 * 2;
-    a.table_in_smem = tab_bytes <= 200 * 1024 ? 1u : 0u;
+    a.table_in_smem = tab_bytes <= kDecodeTableThread ? 1u : 0u;
     a.vector = (hdr->interval % 16 == 0 && ((uintptr_t)d_text & 15) == 0 && ((uintptr_t)d_cols & 15) == 0) ? 1u : 0u;
     const size_t smem = a.table_in_smem ? tab_bytes : 0;
     cudaStream_t s = (cudaStream_t)stream;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(slpf_dfa_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
-        if (e != cudaSuccess) { set_error(std::string("decode attribute: ") + cudaGetErrorString(e)); return RE_E_CUDA; }
-    }
     slpf_dfa_status_kernel<<<1, 1, 0, s>>>(d_status);
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -542,6 +542,8 @@ extern "C" re_status re_slpf_dfa_decode(const re_slpf_dfa_header *hdr, const voi
         if (e != cudaSuccess) { set_error(std::string("decode launch: ") + cudaGetErrorString(e)); return RE_E_CUDA; }
         return RE_OK;
     }
+    static uint64_t attr_done = 0;
+    allow_smem(slpf_dfa_decode_kernel, &attr_done, kDecodeTableThread);
     const uint64_t want = (hdr->n_checkpoints + 255) / 256;
     const uint32_t blocks = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * 4));
     slpf_dfa_decode_kernel<<<blocks, 256, smem, s>>>(a);
