@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kern
     if (staged) {
         for (uint32_t q = threadIdx.x; q < rows * 256; q += blockDim.x) {
             const uint32_t b = q & 255, v = __ldg(a.table + q);
-            if (used[b]) tab[(q >> 8) * rowe + cls[b]] = v == kNoEntry ? (Entry)none : (Entry)v;
+            if (used[b]) tab[(q >> 8) * rowe + cls[b]] = v >= rows ? (Entry)none : (Entry)v;   // kNoEntry, or no id
         }
         for (uint32_t q = threadIdx.x; q < rows; q += blockDim.x) tab[q * rowe + nc - 1] = (Entry)none;
     }
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kern
     auto next_of = [&](uint32_t cur, uint32_t byte) -> uint32_t {   // none: no such pair in the archived text
         if (staged) return tab[cur * rowe + cls[byte]];
         const uint32_t v = __ldg(a.table + (size_t)cur * 256 + byte);
-        return v == kNoEntry ? none : v;
+        return v >= rows ? none : v;
     };
     bool bad = false;
     for (uint64_t w = (uint64_t)blockIdx.x * decode_warps<CB>() + warp; w < a.n_checkpoints * windows;
