@@ -223,7 +223,14 @@ constexpr uint32_t kWindow = 4096;
 template <int CB> constexpr uint32_t decode_warps() { return CB == 1 ? 28u : CB == 2 ? 16u : 8u; }   // what the shared memory holds
 constexpr uint32_t kDecodeExc = 512;           // exceptions staged per window; the rest are read from the archive
 constexpr uint32_t kDecodeTable = 48 * 1024;   // table bytes staged at most
-constexpr uint32_t kDecodeMinInterval = 256;
+constexpr uint32_t kDecodeRows = 192;          // rows looked through for staging, or in long texts
+constexpr uint32_t kDecodeRowsLong = 400;      // as many as a thread-per-piece block stages
+constexpr uint32_t kDecodeMinInterval = 256;   // shorter pieces: a thread each
+// Below kDecodeShort a thread each, too, from kDecodePieces * K pieces on: a warp's lanes then
+// have 8 to 16 columns each, and copying the tile weighs more than the chains.  Log text, K = 256:
+// 1 MiB 37 us by warps, 85 by threads; 8 MiB 127 and 87; 48 MiB 589 and 268.
+constexpr uint32_t kDecodeShort = 512;
+constexpr uint64_t kDecodePieces = 64;
 
 template <int CB> struct IdOf;
 template <> struct IdOf<1> { using type = uint8_t; };
@@ -243,11 +250,15 @@ __global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kern
     __shared__ uint32_t used[256];
     __shared__ uint8_t cls[256];               // byte -> column of the staged table
     __shared__ uint32_t ncol;
-    // used byte columns: one entry of a row that occurs
+    // Used byte columns: one entry of a row that occurs.  Every block looks the table through,
+    // which pays only where it is small for the columns that follow; else the walk reads it
+    // where it is.  DNA (349 ids, K = 4096): 1 MiB 97 us staged, 66 not; 48 MiB 291 and 328.
+    // 5000 ids, 4 MiB: 472 and 116; 65 534 ids: 3250 and 381.
+    const uint32_t rows = a.n_ids;
+    const bool small = rows <= kDecodeRows || (rows <= kDecodeRowsLong && a.n >= (uint64_t)rows << 16);
     for (uint32_t q = threadIdx.x; q < 256; q += blockDim.x) used[q] = 0;
     __syncthreads();
-    const uint32_t rows = a.n_ids;
-    for (uint32_t q = threadIdx.x; q < rows * 128; q += blockDim.x) {
+    for (uint32_t q = threadIdx.x; small && q < rows * 128; q += blockDim.x) {
         const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(a.table) + q);
         if ((v & 0xFFFFu) != kNoEntry) used[2 * (q & 127)] = 1;
         if (v >> 16 != kNoEntry) used[2 * (q & 127) + 1] = 1;
@@ -268,7 +279,7 @@ __global__ void __launch_bounds__(decode_warps<CB>() * 32, 1) slpf_dfa_warp_kern
     // last column is that of every byte that does not occur
     const uint32_t nc = ncol + 1;
     const uint32_t rowe = ((nc * sizeof(Entry) + 3) / 4 | 1) * 4 / sizeof(Entry);
-    const bool staged = (uint64_t)rows * rowe * sizeof(Entry) <= table_bytes;
+    const bool staged = small && (uint64_t)rows * rowe * sizeof(Entry) <= table_bytes;
     Entry *tab = reinterpret_cast<Entry *>(sm);
     if (staged) {
         for (uint32_t q = threadIdx.x; q < rows * 256; q += blockDim.x) {
@@ -534,7 +545,9 @@ extern "C" re_status re_slpf_dfa_decode(const re_slpf_dfa_header *hdr, const voi
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (hdr->interval >= kDecodeMinInterval) {                 // a warp per piece
+    const bool thread_each = hdr->interval < kDecodeMinInterval ||
+                             (hdr->interval < kDecodeShort && a.vector && hdr->n_checkpoints > kDecodePieces * hdr->interval);
+    if (!thread_each) {                                        // a warp per piece
         cudaError_t e;
         if (col_bytes == 1) e = hdr->n_ids < 255 ? launch_decode_warp<1, true>(a, s, sms) : launch_decode_warp<1, false>(a, s, sms);
         else if (col_bytes == 2) e = hdr->n_ids < 255 ? launch_decode_warp<2, true>(a, s, sms) : launch_decode_warp<2, false>(a, s, sms);
