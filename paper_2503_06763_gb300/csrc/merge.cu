@@ -676,7 +676,7 @@ __device__ __forceinline__ void merge_group(const Params &p, const Tabs &T, cons
     constexpr uint32_t ROWB = 64 * bytes_of(E);
     if (g >= p.Gc) return;
     if (!ok) {                                                // rejected text: every column is empty
-        if (TMA && g < p.Gfast) {
+        if (g < p.Gfast) {
 #pragma unroll
             for (int v = 0; v < (int)(ROWB / 16); ++v) out.put(v, make_uint4(0, 0, 0, 0));
         } else {
