@@ -208,7 +208,7 @@ bool mat_for(const re_handle *h, const re_parse_opts *opts) {
     return mat_capable(h) && !(opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY));
 }
 
-Layout layout_for(const re_handle *h, uint64_t n, uint32_t k, bool mat) {
+Layout layout_for(const re_handle *h, uint64_t n, uint32_t k, bool mat, bool batch_walk = false) {
     Layout L{};
     L.k = k;
     L.c = (uint32_t)((n + k - 1) / k);
@@ -230,10 +230,12 @@ Layout layout_for(const re_handle *h, uint64_t n, uint32_t k, bool mat) {
         scan_join(h) ? 2 * c * 4 : 0, scan_join(h) ? 2 * c * 4 : 0,   // fLink, bLink
         kScanWords * 4,
         mat ? (size_t)n + 1 + 128 : 0, mat ? (size_t)n + 1 + 128 : 0};   // FS, BS (one byte per column)
+    // The lane walk of a batch has no use for checkpoints, records and the scan's maps and links.
+    auto unused = [&](int j) { return batch_walk && (j == 4 || j == 5 || (j >= 14 && j <= 17) || (j >= 19 && j <= 22)); };
     size_t o = 0;
     for (int j = 0; j < kArrays; ++j) {
         L.off[j] = o;
-        o += align256(sizes[j] ? sizes[j] : 4);
+        o += unused(j) ? 0 : align256(sizes[j] ? sizes[j] : 4);
     }
     L.total = o;
     return L;
@@ -949,17 +951,22 @@ struct re_batch {
 namespace slpf {
 namespace {
 
-// Chunk length of one text of a batch.  Lane walk: the bytes of all its groups
-// over twice the lanes of a direction (a warp then takes about two tiles from
-// the queue), and a length that makes the text's chunks whole tiles of 32.
-// Otherwise the single-text rule applied to the group's total bytes (one reach
-// lane per chunk, about one wave of lanes for the whole group), but short
-// enough that the text spans a warp tile of 32 chunks where it can.
-uint32_t batch_chunk(const re_handle *h, uint64_t len, uint64_t group_bytes, bool walk, bool recognize, int sms,
+// Chunk length of one text of a batch: the bytes of its group over the lanes
+// of plain_chunk, but short enough that the text spans a warp tile of 32 chunks
+// where it can.  Lane walk: longer where the bytes of all its groups
+// (walk_bytes) over twice the lanes of a direction are (a warp then takes about
+// two tiles from the queue), and a length that makes the text's chunks whole
+// tiles.  Without the group's own bound a batch of one RE had twice the chunks
+// and up to three times the workspace, and was slower: log text, 64 MiB, 205 us
+// with 704-byte chunks and 172 with 1152, recognized 105 (384) and 83.
+uint32_t batch_chunk(const re_handle *h, uint64_t len, uint64_t group_bytes, uint64_t walk_bytes, bool recognize, int sms,
                      const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
-    const uint64_t kg = chunk_for(group_bytes, walk ? 2 * walk_lanes(h->dev, recognize, sms) : (uint64_t)sms * 384);
-    const uint64_t tiles = walk ? std::max<uint64_t>(1, (len + 32 * kg - 1) / (32 * kg)) : 1;
+    uint64_t kg = plain_chunk(group_bytes, sms), tiles = 1;
+    if (walk_bytes) {
+        kg = std::max<uint64_t>(kg, chunk_for(walk_bytes, 2 * walk_lanes(h->dev, recognize, sms)));
+        tiles = std::max<uint64_t>(1, (len + 32 * kg - 1) / (32 * kg));
+    }
     uint64_t kt = (len + 32 * tiles - 1) / (32 * tiles);
     kt = (kt + kSub - 1) / kSub * kSub;
     return (uint32_t)std::max<uint64_t>(256, std::min<uint64_t>(kg, kt));
@@ -1160,9 +1167,9 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
     for (uint32_t j = 0; j < count; ++j) {
         re_batch::Text &t = b->texts[j];
         const re_batch::Group &tg = b->groups[t.group];
-        t.k = batch_chunk(tg.h, t.len, tg.walk ? walk_bytes : gbytes[t.group], tg.walk, b->recognize, b->sms, opts);
+        t.k = batch_chunk(tg.h, t.len, gbytes[t.group], tg.walk ? walk_bytes : 0, b->recognize, b->sms, opts);
         if (t.len / t.k >= 0xFFFFFFF0ull) { set_error("text too long for this chunk length"); return RE_E_INVALID_ARG; }
-        if (t.len) t.L = layout_for(b->groups[t.group].h, t.len, t.k, mat_capable(tg.h) && !b->recognize);
+        if (t.len) t.L = layout_for(tg.h, t.len, t.k, mat_capable(tg.h) && !b->recognize, tg.walk);
     }
     uint32_t slot = 0;                                       // every text's Params, group after group
     for (auto &g : b->groups) {
@@ -1201,7 +1208,7 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
         }
     }
     plan_walk(b.get(), gbytes);
-    b->wgroups_off = off; off = align256(off + b->groups.size() * sizeof(WalkGroup));
+    b->wgroups_off = off; off = align256(off + (b->wb.n_heads ? b->groups.size() * sizeof(WalkGroup) : 0));
     b->heads_off = off; off = align256(off + b->heads.size() * sizeof(WalkSpan));
     b->walk_off = off; off = align256(off + b->walk.size() * sizeof(WalkSpan));
     b->gather_off = off; off = align256(off + b->gather.size() * sizeof(WalkSpan));
@@ -1322,7 +1329,7 @@ re_status re_parse_batch(re_batch *b, const uint8_t *const *d_texts, re_slpf *ou
     }
     for (size_t j = 0; j < b->groups.size(); ++j) {          // the lane-walk groups' descriptors
         const re_batch::Group &g = b->groups[j];
-        if (!g.walk) continue;
+        if (!g.walk || !b->wb.n_heads) continue;
         WalkGroup d{};
         d.t = g.h->dev;
         d.texts = reinterpret_cast<const Params *>(w + g.params_off);
