@@ -512,8 +512,8 @@ __device__ void join_walk_fix(const Params &p, const LaneTab &T, uint32_t ns, ui
     const uint32_t in = __ldcg(J + (FWD ? i : i + 1)), out = __ldcg(J + (FWD ? i + 1 : i));
     bool fail = in == 0 || out == 0 || out >= ns;
     if (OUT && FWD && i == p.c - 1) S[p.n] = (uint8_t)out;
-    if (!fail && (FWD ? i + 1 < p.c : i > 0)) {
-        const uint32_t o = FWD ? i + 1 : i - 1;
+    const uint32_t o = FWD ? i + 1 : i - 1;
+    if (!fail && (FWD ? i + 1 < p.c : i > 0) && (OUT || kinds[o] == 0)) {   // else no columns, and no state to check
         const uint64_t nbase = (uint64_t)o * p.k;
         const uint32_t nlen = chunk_len(p, o), edge = min(kUnit * (FWD ? p.w.fconv : p.w.bconv)[o], nlen);
         uint32_t mid;

@@ -131,6 +131,7 @@ __device__ bool walk_chunk(const Params &p, const LaneTab &T, uint32_t ns, uint6
     // columns of the next chunk's head
     auto head_of = [&]() -> uint32_t {
         if (!known || p.rall || !(FWD ? i + 1 < p.c : i > 0)) return 0;
+        if (!OUT && kinds[o] != 0) return 0;                  // no columns, and no state to check
         const uint32_t nlen = chunk_len(p, o), e = min(kUnit * convs[o], nlen);
         return FWD ? e : nlen - e;
     };
