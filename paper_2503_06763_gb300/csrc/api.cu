@@ -84,11 +84,6 @@ uint32_t plain_chunk(uint64_t n, int sms) { return chunk_for(n, (uint64_t)sms * 
 // at once (8 blocks of 64 per SM) while chunks are below 384 bytes, as a head
 // costs about as much as 100 bytes of walk (11 MiB of log text: 320 take 47 us
 // where 256 take 55; 12.5 MiB: 384 49, 256 64).
-// A recognizer has one direction's chunks to walk and as many to join: those of
-// plain_chunk, more (as many as the device takes heads at once) where they stay
-// above 1152 bytes.  Log text: 24 MB 49 us with 320 to 512, 64 MiB 70 with 1152 and
-// 72 with 704, 256 MiB 149 with 3456 and 173 with 4608; 64 MiB in one line, whose
-// runs never meet, 1349 us with 704 and 904 with 1152.
 // Warp pairs: the chunks of plain_chunk, or fewer where half of them or less
 // are better: a chunk's bytes are walked one after another, 24 ns each, and
 // each chunk costs the join about 4 ns when byte states make it a scan over all
@@ -99,12 +94,11 @@ uint32_t plain_chunk(uint64_t n, int sms) { return chunk_for(n, (uint64_t)sms * 
 uint32_t choose_chunk(const re_handle *h, uint64_t n, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
     const bool rec = opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY);
-    const uint64_t most = (uint64_t)sms * 384;
     if (walk_first(h)) {
         const uint64_t heads = (uint64_t)sms * 8 * 64 / (rec ? 1 : 2);
-        if (rec) return chunk_for(n, std::max(most, std::min(n / 1152, heads)));
         return chunk_for(n, std::max(heads, std::min(n / 384, walk_lanes(h->dev, rec, sms))));
     }
+    const uint64_t most = (uint64_t)sms * 384;
     const uint64_t fewer = std::max<uint64_t>(1, (uint64_t)std::sqrt((scan_join(h) ? 8.0 : 16.0) * (double)n));
     return chunk_for(n, fewer <= most / 2 ? fewer : most);
 }
