@@ -265,6 +265,13 @@ re_status resolve_kind(const re_handle *h, re_slpf_kind kind, re_slpf_kind &out,
     return RE_OK;
 }
 
+// Chunks per unit of the join's scan: more of them are composed one after another
+// by a warp, fewer units take their rounds.  Join of runs that never meet, us:
+// (aa)* 16 MiB (11 398 chunks) 223 with 1, 127 with 4, 123 with 8; one line under
+// the log RE, 64 MiB (58 255) 1360, 695, 679, and 16 MiB (37 450) 938, 457, 393; but
+// the genome RE, whose chains are short, 4 MiB (5793) 55, 86, 68.
+uint32_t scan_group(uint32_t c) { return c < 8192 ? 1u : c < 32768 ? 4u : 8u; }
+
 // True for device (or managed) memory; false for host memory the device
 // reaches over the host link (pinned, mapped).
 bool in_device_memory(const void *ptr) {
@@ -575,7 +582,7 @@ re_status slpf::parse_impl(re_handle *h, const uint8_t *d_text, uint64_t len, re
     p.out = recognize ? nullptr : slpf->d_cols;
     p.col_bytes = cb; p.kind = kind; p.status = slpf->d_status;
     p.recognize = (recognize && !map_mode) ? 1u : 0u;          // map mode walks both directions
-    p.scan = scan_join(h) ? 1u : 0u;
+    p.scan = scan_join(h) ? scan_group(L.c) : 0u;
     p.scan_stall = (opts && (opts->flags & RE_PARSE_TEST_STALL_JOIN)) ? 1u : 0u;
     const DevTables &t = h->dev;
     p.tmode = table_mode(t);

@@ -420,75 +420,126 @@ __device__ bool grid_barrier(uint32_t *w) {
     return ok != 0;
 }
 
-// One direction of one chunk in a round.  LANES = 32: a warp, whose lanes
-// share the table work; LANES = 1: one thread (small automata, where the
-// latency of the link reads, not the table, sets the time of a round).
-template <bool FWD, uint32_t LANES>
-__device__ uint32_t scan_step(const Params &p, uint32_t i, uint32_t cur) {
-    const uint32_t lane = LANES == 1 ? 0u : (threadIdx.x & 31), c = p.c, ns = (FWD ? p.t.nfd : p.t.nbd) + 1;
+// The scan's units are groups of p.scan consecutive chunks (at most 32): a warp
+// composes a group's maps, its lanes over the states, and once the scan has every
+// group's output, a thread per group takes the state through its chunks.  In a
+// round a unit costs its barrier's share and two dependent reads whatever it
+// stands for, so tens of thousands of single chunks were most of the join: 64 MiB in
+// one line under the log RE 1360 us with a unit per chunk, 679 with one per 8.
+template <bool FWD> struct ScanGroup {
+    uint32_t a, n;                                     // its first chunk in the text, and how many
+    __device__ ScanGroup(const Params &p, uint32_t g) : a(g * p.scan), n(min(p.scan, p.c - g * p.scan)) {}
+    __device__ uint32_t chunk(uint32_t q) const { return FWD ? a + q : a + n - 1 - q; }   // in walking order
+    __device__ uint32_t in() const { return FWD ? a : a + n; }      // J indices of its input and output
+    __device__ uint32_t out() const { return FWD ? a + n : a; }
+};
+
+// A group whose output some chunk of its own determines is resolved at once;
+// the others get their map over the classic-DFA states.
+template <bool FWD>
+__device__ void scan_map(const Params &p, uint32_t g, bool &bad) {
+    const uint32_t lane = threadIdx.x & 31, ns = (FWD ? p.t.nfd : p.t.nbd) + 1;
+    const ScanGroup<FWD> G(p, g);
+    uint32_t *J = FWD ? p.w.FJ : p.w.BJ, *link = FWD ? p.w.fLink : p.w.bLink;
+    const uint32_t *kinds = FWD ? p.w.fkind : p.w.bkind;
+    const unsigned known = __ballot_sync(0xFFFFFFFFu, lane < G.n && kinds[G.chunk(lane < G.n ? lane : 0)] == 0);
+    if (known) {
+        if (lane == 0) {
+            uint32_t q = 31 - __clz(known);            // the last of them
+            if (q + 1 < G.n) {
+                uint32_t cur = J[FWD ? G.chunk(q) + 1 : G.chunk(q)];
+                while (++q < G.n) cur = eval_chunk(p, FWD, G.chunk(q), cur, bad);
+                J[G.out()] = cur;
+            }
+            link[g] = kResolved;
+        }
+        return;
+    }
+    uint8_t *T = (FWD ? p.w.fTab : p.w.bTab) + (size_t)g * ns;
+    for (uint32_t S = lane; S < ns; S += 32) {
+        uint32_t cur = S;
+        for (uint32_t q = 0; q < G.n; ++q) cur = eval_chunk(p, FWD, G.chunk(q), cur, bad);
+        T[S] = (uint8_t)cur;
+    }
+    if (lane == 0) link[g] = FWD ? g - 1 : g + 1;      // the text's first (last) chunk has one output
+}
+
+// One direction of one group in a round, by a warp.
+template <bool FWD>
+__device__ uint32_t scan_step(const Params &p, uint32_t g, uint32_t ng, uint32_t cur) {
+    const uint32_t lane = threadIdx.x & 31, ns = (FWD ? p.t.nfd : p.t.nbd) + 1;
     uint32_t *link = FWD ? p.w.fLink : p.w.bLink;
     uint8_t *tab = FWD ? p.w.fTab : p.w.bTab;
     uint32_t *J = FWD ? p.w.FJ : p.w.BJ;
     const uint32_t nxt = cur ^ 1u;
-    const uint32_t l = __ldcg(link + (size_t)cur * c + i);
+    const uint32_t l = __ldcg(link + (size_t)cur * ng + g);
     if (l == kResolved) {
-        if (lane == 0) link[(size_t)nxt * c + i] = kResolved;
+        if (lane == 0) link[(size_t)nxt * ng + g] = kResolved;
         return 0;
     }
-    const uint8_t *Ti = tab + ((size_t)cur * c + i) * ns;
-    const uint32_t ll = __ldcg(link + (size_t)cur * c + l);
+    const uint8_t *Tg = tab + ((size_t)cur * ng + g) * ns;
+    const uint32_t ll = __ldcg(link + (size_t)cur * ng + l);
     if (ll == kResolved) {                             // the range's input is known
         if (lane == 0) {
-            const uint32_t v = __ldcg(J + (FWD ? l + 1 : l));   // output of chunk l
-            J[FWD ? i + 1 : i] = v < ns ? (uint32_t)__ldcg(Ti + v) : 0u;   // v >= ns: no DFA state, rejected
-            link[(size_t)nxt * c + i] = kResolved;
+            const uint32_t v = __ldcg(J + ScanGroup<FWD>(p, l).out());
+            J[ScanGroup<FWD>(p, g).out()] = v < ns ? (uint32_t)__ldcg(Tg + v) : 0u;   // v >= ns: no DFA state, rejected
+            link[(size_t)nxt * ng + g] = kResolved;
         }
         return 0;
     }
-    const uint8_t *Tl = tab + ((size_t)cur * c + l) * ns;
-    uint8_t *Tn = tab + ((size_t)nxt * c + i) * ns;
-    for (uint32_t S = lane; S < ns; S += LANES) Tn[S] = __ldcg(Ti + __ldcg(Tl + S));
-    if (lane == 0) link[(size_t)nxt * c + i] = ll;
+    const uint8_t *Tl = tab + ((size_t)cur * ng + l) * ns;
+    uint8_t *Tn = tab + ((size_t)nxt * ng + g) * ns;
+    for (uint32_t S = lane; S < ns; S += 32) Tn[S] = __ldcg(Tg + __ldcg(Tl + S));
+    if (lane == 0) link[(size_t)nxt * ng + g] = ll;
     return 1;
 }
 
-// False when a barrier wait ran out.
-template <uint32_t LANES>
-__device__ bool join_scan(const Params &p) {
-    const uint32_t lane = LANES == 1 ? 0u : (threadIdx.x & 31), upb = blockDim.x / LANES;
-    const uint64_t gw = (uint64_t)blockIdx.x * upb + threadIdx.x / LANES, nw = (uint64_t)gridDim.x * upb;
-    const bool bwd = !p.recognize;
-    // maps of the chunks whose output depends on their input
-    bool bad = false;
-    for (uint64_t i = gw; i < p.c; i += nw) {
-        if (p.w.fkind[i]) {                           // i >= 1: chunk 0 always has one output
-            uint8_t *T = p.w.fTab + i * (p.t.nfd + 1);
-            for (uint32_t S = lane; S <= p.t.nfd; S += LANES)
-                T[S] = (uint8_t)eval_chunk(p, true, (uint32_t)i, S, bad);
-        }
-        if (lane == 0) p.w.fLink[i] = p.w.fkind[i] ? (uint32_t)i - 1 : kResolved;
-        if (!bwd) continue;
-        if (p.w.bkind[i]) {                           // i <= c-2
-            uint8_t *T = p.w.bTab + i * (p.t.nbd + 1);
-            for (uint32_t S = lane; S <= p.t.nbd; S += LANES)
-                T[S] = (uint8_t)eval_chunk(p, false, (uint32_t)i, S, bad);
-        }
-        if (lane == 0) p.w.bLink[i] = p.w.bkind[i] ? (uint32_t)i + 1 : kResolved;
+// The states between a group's chunks from its input, by a thread.
+template <bool FWD>
+__device__ void scan_fill(const Params &p, uint32_t g, bool &bad) {
+    const ScanGroup<FWD> G(p, g);
+    uint32_t *J = FWD ? p.w.FJ : p.w.BJ;
+    const uint32_t *kinds = FWD ? p.w.fkind : p.w.bkind;
+    uint32_t cur = __ldcg(J + G.in());
+    for (uint32_t q = 0; q < G.n; ++q) {
+        const uint32_t i = G.chunk(q);
+        uint32_t *o = J + (FWD ? i + 1 : i);
+        if (kinds[i]) *o = cur = eval_chunk(p, FWD, i, cur, bad);
+        else cur = __ldcg(o);
     }
-    if (bad) atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
+}
+
+// False when a barrier wait ran out.
+__device__ bool join_scan(const Params &p) {
+    const uint32_t wpb = blockDim.x / 32, ng = (p.c + p.scan - 1) / p.scan;
+    const uint64_t gw = (uint64_t)blockIdx.x * wpb + threadIdx.x / 32, nw = (uint64_t)gridDim.x * wpb;
+    const bool bwd = !p.recognize;
+    bool bad = false;
+    for (uint64_t g = gw; g < ng; g += nw) {
+        scan_map<true>(p, (uint32_t)g, bad);
+        if (bwd) scan_map<false>(p, (uint32_t)g, bad);
+    }
     if (p.scan_stall && blockIdx.x == 0) return false;   // test hook: the other blocks' waits run out
     if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return false; }
     for (uint32_t r = 0; r < kScanRounds; ++r) {
         uint32_t open = 0;
-        for (uint64_t i = gw; i < p.c; i += nw) {
-            open += scan_step<true, LANES>(p, (uint32_t)i, r & 1);
-            if (bwd) open += scan_step<false, LANES>(p, (uint32_t)i, r & 1);
+        for (uint64_t g = gw; g < ng; g += nw) {
+            open += scan_step<true>(p, (uint32_t)g, ng, r & 1);
+            if (bwd) open += scan_step<false>(p, (uint32_t)g, ng, r & 1);
         }
-        if (LANES == 1) open = __reduce_add_sync(0xFFFFFFFFu, open);
         if ((threadIdx.x & 31) == 0 && open) atomicAdd(p.w.scan + 2 + r, open);
         if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return false; }
-        if (__ldcg(p.w.scan + 2 + r) == 0) break;     // every chunk resolved (same value in every block)
+        if (__ldcg(p.w.scan + 2 + r) == 0) break;     // every group resolved (same value in every block)
     }
+    if (bad) atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
+    if (p.scan == 1) return true;                     // a group's output is its chunk's
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < (bwd ? 2ull : 1ull) * ng;
+         j += (uint64_t)gridDim.x * blockDim.x) {
+        if (j < ng) scan_fill<true>(p, (uint32_t)j, bad);
+        else scan_fill<false>(p, (uint32_t)(j - ng), bad);
+    }
+    if (bad) atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
+    if (!grid_barrier(p.w.scan)) { atomicExch(&p.w.flags[FLAG_TIMEOUT], 1); return false; }
     return true;
 }
 
@@ -496,8 +547,7 @@ __global__ void __launch_bounds__(kBlockThreads) join_scan_kernel(const __grid_c
     // every chunk has one output for every input (the common case): classify
     // has resolved them all
     if (__ldcg(p.w.scan + kScanGeneral) == 0 && !p.scan_stall) return;
-    if (p.t.nfd < 16 && p.t.nbd < 16) join_scan<1>(p);   // tables of at most 16 entries: a thread per chunk
-    else join_scan<32>(p);
+    join_scan(p);
 }
 
 // ------------------------------------------------------------------ after the lane walk
@@ -537,8 +587,7 @@ __global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_c
         if (blockIdx.x == 0 && threadIdx.x == 0) status_of(p);
         return;
     }
-    const bool ok = p.t.nfd < 16 && p.t.nbd < 16 ? join_scan<1>(p) : join_scan<32>(p);
-    if (!ok) {
+    if (!join_scan(p)) {
         if (threadIdx.x == 0) atomicExch(p.status, RE_E_TIMEOUT);
         return;
     }
@@ -637,14 +686,14 @@ __global__ void batch_init_kernel(const Params *texts, uint32_t nt, uint32_t *qu
 
 }  // namespace
 
-// Cooperative launch of kernel with a warp (or a thread) per chunk, at most
-// the blocks the device holds at once.
+// Cooperative launch of kernel with a warp per unit, at most the blocks the
+// device holds at once.
 template <typename... KArgs, typename... Args>
-static bool launch_coop(void (*kernel)(KArgs...), size_t smem, uint64_t chunks, cudaStream_t s, int sm_count,
+static bool launch_coop(void (*kernel)(KArgs...), size_t smem, uint64_t units, cudaStream_t s, int sm_count,
                         Args &&...args) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlockThreads, smem);
-    const uint64_t want = (chunks + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
+    const uint64_t want = (units + kBlockThreads / 32 - 1) / (kBlockThreads / 32);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)std::max(per_sm, 1) * sm_count));
     cfg.blockDim = kBlockThreads;
@@ -658,13 +707,17 @@ static bool launch_coop(void (*kernel)(KArgs...), size_t smem, uint64_t chunks, 
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) == cudaSuccess;
 }
 
+// A warp per group of the scan, and a second block where there are chunks for
+// one (the bounded waits are tested between blocks).
+static uint64_t scan_units(const Params &p) { return std::max(p.c / p.scan + 1, std::min(p.c, 16u)); }
+
 // Classify, then the scan (a cooperative launch: its blocks meet at grid
 // barriers, so they must all be resident) or the chains, then verify.
 bool launch_join(const Params &p, cudaStream_t s, int sm_count) {
     const uint32_t blocks = (p.c + kBlockThreads - 1) / kBlockThreads;
     launch_dependent(join_classify_kernel, blocks, kBlockThreads, 0, s, p);
     if (p.scan) {
-        if (!launch_coop(join_scan_kernel, 0, p.c, s, sm_count, p)) return false;
+        if (!launch_coop(join_scan_kernel, 0, scan_units(p), s, sm_count, p)) return false;
     } else {
         launch_dependent(join_chain_kernel, blocks, kBlockThreads, 0, s, p);
     }
@@ -693,7 +746,7 @@ bool launch_join_walk(const Params &p, cudaStream_t s, int sm_count) {
     const size_t smem = join_walk_smem(p.t);
     static uint64_t attr_done = 0;
     allow_smem(join_walk_kernel, &attr_done);
-    return launch_coop(join_walk_kernel, smem, p.c, s, sm_count, p);
+    return launch_coop(join_walk_kernel, smem, scan_units(p), s, sm_count, p);
 }
 
 // A slice's maps after the lane walk (every slot's end state, p.rall) or the

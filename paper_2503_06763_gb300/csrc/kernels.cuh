@@ -36,7 +36,7 @@ enum { SHARD_PREV = 1, SHARD_NEXT = 2 };
 // at most kScanStates states (ids fit a byte), so a chunk's map over them is
 // a byte table.
 constexpr uint32_t kScanStates = 256;
-constexpr uint32_t kScanRounds = 40;        // pointer-jumping rounds (chains up to 2^40 chunks)
+constexpr uint32_t kScanRounds = 40;        // pointer-jumping rounds (chains up to 2^40 units)
 constexpr uint32_t kScanWords = 64;         // barrier words + per-round counters
 constexpr uint32_t kScanGeneral = 2 + kScanRounds;   // scan word: chunks whose output depends on their input
 
@@ -54,8 +54,8 @@ struct Work {                       // device workspace, carved from the caller'
     uint2 *recFe, *recBe;           // [c][kRecEntries] (state, slot set) of those runs
     int32_t *flags;                 // [FLAG_COUNT]
     uint8_t *FS, *BS;               // [n+1+pad] per-position forward / backward states (mat), one byte each
-    uint8_t *fTab, *bTab;           // [2][c][nfd+1], [2][c][nbd+1]: maps of chunk ranges (scan join)
-    uint32_t *fLink, *bLink;        // [2][c]: chunk whose output feeds the range's map (scan join)
+    uint8_t *fTab, *bTab;           // [2][c][nfd+1], [2][c][nbd+1]: maps of unit ranges (scan join)
+    uint32_t *fLink, *bLink;        // [2][c]: unit whose output feeds the range's map (scan join)
     uint32_t *scan;                 // [kScanWords]: grid barrier and per-round counters (scan join)
 };
 
@@ -70,7 +70,8 @@ struct Params {
     uint32_t col_bytes, kind;       // output encoding (re_slpf_kind)
     int32_t *status;
     uint32_t recognize;             // forward reach + join only
-    uint32_t scan;                  // join by the pointer-jumping scan (else chains, one thread each)
+    uint32_t scan;                  // join by the pointer-jumping scan, in units of this many chunks; 0: by
+                                    // chains, one thread each
     uint32_t scan_stall;            // test hook: one block of the scan never reaches its first barrier
     uint32_t mat;                   // reach writes every position's state once its runs have met; the
                                     // fix-up fills the positions before; build & merge is a gather
