@@ -597,13 +597,15 @@ __global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_c
     stage_lane_table<0>(p.t.bc8, nsb * cw, sm + 256 + nsf * cw * 4);
     __syncthreads();
     const LaneTab F{smem_u32(sm + 256), sm, cw * 4}, B{smem_u32(sm + 256 + nsf * cw * 4), sm, cw * 4};
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.c; i += (uint64_t)gridDim.x * blockDim.x) {
-        if (p.mat) {
-            join_walk_fix<true, true>(p, F, nsf, (uint32_t)i);
-            join_walk_fix<false, true>(p, B, nsb, (uint32_t)i);
+    const uint64_t items = (p.recognize ? 1ull : 2ull) * p.c;     // a thread per chunk and direction
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < items; j += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = (uint32_t)(j < p.c ? j : j - p.c);
+        if (j < p.c) {
+            if (p.mat) join_walk_fix<true, true>(p, F, nsf, i);
+            else join_walk_fix<true, false>(p, F, nsf, i);
         } else {
-            join_walk_fix<true, false>(p, F, nsf, (uint32_t)i);
-            if (!p.recognize) join_walk_fix<false, false>(p, B, nsb, (uint32_t)i);
+            if (p.mat) join_walk_fix<false, true>(p, B, nsb, i);
+            else join_walk_fix<false, false>(p, B, nsb, i);
         }
     }
     if (!grid_barrier(p.w.scan)) {
