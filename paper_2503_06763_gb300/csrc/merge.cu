@@ -182,6 +182,7 @@ constexpr uint32_t kFixItems = 32;
 struct FixShared {
     uint32_t chunk[kFixItems], text[kFixItems], nrec[kFixItems], H[kFixItems], conv[kFixItems];
     uint32_t walk[kFixItems];                 // 1: boundaries past the record remain (after record nrec-1)
+    uint32_t from[kFixItems];                 // the state at the last record
     uint32_t first[kFixItems + 1];            // flat index of each item's first record
     uint32_t off[kFixItems][kRecBounds];      // entry offset of each record in its item's row
     uint32_t cnt[kFixItems][kRecBounds];      // entries of each record
@@ -292,11 +293,13 @@ __device__ void fix_block(const Tabs &T, FixShared &S, RF R, PF P) {
             const uint32_t nsub = (chunk_len(p, (uint32_t)i) + 63) / 64;
             p.w.BC[g0 + (nsub - 1 - r) - 1] = st;               // record r: boundary nsub-1-r
         }
-        if (r + 1 == S.nrec[q] && (S.walk[q] & 1u)) fixup_walk<TM>(p, T, i, fwd, S.nrec[q], S.conv[q], st);
+        if (r + 1 == S.nrec[q]) S.from[q] = st;
     }
-    if (threadIdx.x < kFixItems && S.nrec[threadIdx.x] == 0 && (S.walk[threadIdx.x] & 1u)) {   // walks with no record
+    __syncthreads();
+    // the walks past the records, a lane an item: where no runs meet every item has one
+    if (threadIdx.x < kFixItems && (S.walk[threadIdx.x] & 1u)) {
         const uint32_t q = threadIdx.x;
-        fixup_walk<TM>(P(S.text[q]), T, S.chunk[q], S.walk[q] & 2u, 0u, S.conv[q], 0u);
+        fixup_walk<TM>(P(S.text[q]), T, S.chunk[q], S.walk[q] & 2u, S.nrec[q], S.conv[q], S.from[q]);
     }
     __syncthreads();                                            // S is refilled next
 }
