@@ -31,7 +31,7 @@ constexpr uint32_t kHeadChunks = 64;        // chunks a block takes at once, at 
 constexpr uint32_t kHeadWindow = 144;       // bytes of a chunk staged, from its edge (a multiple of 16)
 constexpr uint32_t kHeadStride = 148;       // their stride: an odd number of words, so lanes hit different banks
 constexpr int kRuns = 4;
-constexpr uint32_t kWideBytes = 64;         // bytes a warp walks a chunk's slots
+constexpr uint32_t kWideBytes = 32;         // bytes a warp walks a chunk's slots
 
 // Drop dead runs and merge runs in equal states (their slot sets are joined);
 // unused runs hold the empty state.
@@ -108,7 +108,7 @@ __device__ __forceinline__ void head_word(const LaneTab &T, uint32_t w, uint32_t
 // where more runs than a lane keeps are apart after kWideBytes.  They hardly
 // ever meet later, so they are not compared; a state is a byte, and the eight are
 // kept in two words.  A warp per chunk walking them on to its end, most of its
-// lanes idle, made the heads of 64 MiB of a's under twenty (c{6}) 3.4 ms; now 0.6.
+// lanes idle, made the heads of 64 MiB of a's under twenty (c{6}) 3.4 ms; now 0.45.
 template <bool FWD>
 __device__ void slots_to_end(const LaneTab &T, const uint8_t *x, uint32_t len, const uint32_t *starts, uint32_t m,
                              uint32_t ms, uint32_t *R) {
