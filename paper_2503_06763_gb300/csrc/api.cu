@@ -1205,6 +1205,7 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
         for (uint32_t j : g.members) {
             const re_batch::Text &t = b->texts[j];
             const uint64_t c = t.len ? t.L.c : 0;
+            if (g.walk && c > kJoinChunks) b->wb.long_texts = 1;
             g.chunks += c;
             g.n_reach += (c + 31) / 32;
             g.n_merge += ((t.len && !b->recognize ? t.L.Gc : 0) + 31) / 32;
@@ -1355,6 +1356,7 @@ re_status re_parse_batch(re_batch *b, const uint8_t *const *d_texts, re_slpf *ou
     b->wb.walk = reinterpret_cast<const WalkSpan *>(w + b->walk_off);
     b->wb.gather = reinterpret_cast<const WalkSpan *>(w + b->gather_off);
     b->wb.texts = reinterpret_cast<const Params *>(w);
+    b->wb.general = reinterpret_cast<uint32_t *>(w + b->queue_off) + 2;   // a word of the first group's counters
     b->wb.nt = count;
     cudaStream_t s = (cudaStream_t)stream;
     CUDA_TRY(cudaMemcpyAsync(w, b->pinned, b->desc_bytes, cudaMemcpyHostToDevice, s), "batch descriptor upload");

@@ -125,16 +125,17 @@ __device__ void classify_at(const Params &p, uint32_t i) {
 
 // Chains of general chunks, evaluated in order from their known neighbour
 // (started by the chunk just after / before the neighbour).
-__device__ void chain_at(const Params &p, uint32_t i) {
+template <bool FWD>
+__device__ void chain_from(const Params &p, uint32_t i) {
     bool bad = false;
-    if (p.w.fkind[i] == 1 && p.w.fkind[i - 1] == 0) {     // i >= 1: fkind[0] == 0
+    if (FWD && p.w.fkind[i] == 1 && p.w.fkind[i - 1] == 0) {     // i >= 1: fkind[0] == 0
         uint32_t cur = p.w.FJ[i];
         for (uint32_t j = i; j < p.c && p.w.fkind[j] == 1; ++j) {
             cur = eval_chunk(p, true, j, cur, bad);
             p.w.FJ[j + 1] = cur;
         }
     }
-    if (!p.recognize && p.w.bkind[i] == 1 && p.w.bkind[i + 1] == 0) {   // i <= c-2: bkind[c-1] == 0
+    if (!FWD && p.w.bkind[i] == 1 && p.w.bkind[i + 1] == 0) {    // i <= c-2: bkind[c-1] == 0
         uint32_t cur = p.w.BJ[i + 1];
         for (int64_t j = i; j >= 0 && p.w.bkind[j] == 1; --j) {
             cur = eval_chunk(p, false, (uint32_t)j, cur, bad);
@@ -142,6 +143,10 @@ __device__ void chain_at(const Params &p, uint32_t i) {
         }
     }
     if (bad) atomicExch(&p.w.flags[FLAG_INTERNAL], 1);
+}
+__device__ void chain_at(const Params &p, uint32_t i) {
+    chain_from<true>(p, i);
+    if (!p.recognize) chain_from<false>(p, i);
 }
 
 __global__ void join_classify_kernel(const __grid_constant__ Params p) {
@@ -554,6 +559,7 @@ __global__ void __launch_bounds__(kBlockThreads) join_scan_kernel(const __grid_c
 // A general chunk (kind 1: its runs never met) of the lane walk, once the scan
 // has its output: the walk had no state to go on with, so the head of the
 // chunk its run enters is walked here, with the check the walk makes.
+constexpr uint32_t kFixThreads = 64;           // a batch's: as many as a heads round has chunks
 template <bool FWD, bool OUT>
 __device__ void join_walk_fix(const Params &p, const LaneTab &T, uint32_t ns, uint32_t i) {
     const uint32_t *kinds = FWD ? p.w.fkind : p.w.bkind, *J = FWD ? p.w.FJ : p.w.BJ;
@@ -615,10 +621,11 @@ __global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_c
     if (blockIdx.x == 0 && threadIdx.x == 0) status_of(p);
 }
 
-// The same for every text of a batch's lane-walk groups, a block per text.
-// Chunks whose runs never met are evaluated in chains (a text of a batch has
-// few chunks).
-__global__ void join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
+// The same for every text of a batch's lane-walk groups, a block per text, its
+// lower half forward and its upper half backward: chunks whose runs never met are
+// evaluated in chains.  Longer texts with such chunks are left to join_long_kernel.
+constexpr uint32_t kJoinThreads = 256;
+__global__ void __launch_bounds__(kJoinThreads) join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
     extern __shared__ __align__(16) uint8_t sm[];
     const Params &p = b.texts[blockIdx.x];
     if (!p.rvar) return;                                      // a group of the other kernels
@@ -627,7 +634,16 @@ __global__ void join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
         return;
     }
     if (p.w.scan[kScanGeneral]) {
-        for (uint32_t i = threadIdx.x; i < p.c; i += blockDim.x) chain_at(p, i);
+        if (p.c > kJoinChunks) {
+            if (threadIdx.x == 0) *b.general = 1;
+            return;
+        }
+        const uint32_t half = b.recognize ? blockDim.x : blockDim.x / 2, t = threadIdx.x % half;
+        const bool fwd = threadIdx.x < half;
+        for (uint32_t i = t; i < p.c; i += half) {
+            if (fwd) chain_from<true>(p, i);
+            else chain_from<false>(p, i);
+        }
         __threadfence();
         const uint32_t cw = class_words(p.t), nsf = p.t.nfd + 1, nsb = p.t.nbd + 1;
         stage_classes(p.t, sm);
@@ -635,18 +651,60 @@ __global__ void join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
         stage_lane_table<0>(p.t.bc8, nsb * cw, sm + 256 + nsf * cw * 4);
         __syncthreads();
         const LaneTab F{smem_u32(sm + 256), sm, cw * 4}, B{smem_u32(sm + 256 + nsf * cw * 4), sm, cw * 4};
-        for (uint32_t i = threadIdx.x; i < p.c; i += blockDim.x) {
-            if (b.recognize) {
-                join_walk_fix<true, false>(p, F, nsf, i);
-            } else {
-                join_walk_fix<true, true>(p, F, nsf, i);
-                join_walk_fix<false, true>(p, B, nsb, i);
-            }
+        for (uint32_t i = t; i < p.c; i += half) {
+            if (b.recognize) join_walk_fix<true, false>(p, F, nsf, i);
+            else if (fwd) join_walk_fix<true, true>(p, F, nsf, i);
+            else join_walk_fix<false, true>(p, B, nsb, i);
         }
         __threadfence();
         __syncthreads();
     }
     if (threadIdx.x == 0) status_of(p);
+}
+
+// Texts of more than kJoinChunks chunks some of whose runs never met: the
+// chains, then (HEADS) the heads after such chunks, over the spans of the heads
+// kernel, a thread per chunk and direction of all groups.  By a block per text one
+// genome text of 64 MiB took 38 ms.  The last item of a text sets its status.
+// Launched only for batches with such long texts.
+template <bool HEADS>
+__global__ void __launch_bounds__(kFixThreads) join_long_kernel(const __grid_constant__ WalkBatch b) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    pdl_wait();
+    if (!__ldcg(b.general)) return;
+    const bool pairs = !b.recognize, backward = pairs && (blockIdx.x & 1);
+    const WalkSpan w = b.heads[pairs ? blockIdx.x >> 1 : blockIdx.x];
+    const WalkGroup &g = b.groups[w.group];
+    const uint32_t cw = class_words(g.t), ns = (backward ? g.t.nbd : g.t.nfd) + 1;
+    const LaneTab T{smem_u32(sm + 256), sm, cw * 4};
+    bool staged = false;
+    for (uint64_t first = (uint64_t)w.idx * kFixThreads; first < g.chunks; first += (uint64_t)w.cnt * kFixThreads) {
+        const uint64_t j = first + threadIdx.x;
+        const uint32_t ti = j < g.chunks ? text_of(g.chunk_base, g.nt, j) : 0u;
+        const Params &p = g.texts[ti];
+        const uint32_t i = (uint32_t)(j - __ldg(g.chunk_base + ti));
+        const bool mine = j < g.chunks && p.c > kJoinChunks && p.w.scan[kScanGeneral] != 0;
+        if (!HEADS) {
+            if (mine && backward) chain_from<false>(p, i);
+            else if (mine) chain_from<true>(p, i);
+            continue;
+        }
+        if (__syncthreads_or(mine) && !staged) {
+            stage_classes(g.t, sm);
+            stage_lane_table<0>(backward ? g.t.bc8 : g.t.fc8, ns * cw, sm + 256);
+            __syncthreads();
+            staged = true;
+        }
+        if (!mine) continue;
+        if (b.recognize) join_walk_fix<true, false>(p, T, ns, i);
+        else if (backward) join_walk_fix<false, true>(p, T, ns, i);
+        else join_walk_fix<true, true>(p, T, ns, i);
+        __threadfence();
+        if ((uint32_t)atomicAdd(&p.w.flags[FLAG_DONE], 1) + 1 == (pairs ? 2u : 1u) * p.c) {
+            __threadfence();
+            status_of(p);
+        }
+    }
 }
 
 // ------------------------------------------------------------------ batch
@@ -739,9 +797,15 @@ size_t join_walk_smem(const DevTables &t) { return 256 + (size_t)(t.nfd + t.nbd 
 
 void launch_join_walk_batch(const WalkBatch &b, cudaStream_t s) {
     if (!b.nt) return;
-    static uint64_t attr_done = 0;
-    allow_smem(join_walk_batch_kernel, &attr_done);
-    join_walk_batch_kernel<<<b.nt, 128, b.join_smem, s>>>(b);
+    static uint64_t attr_walk = 0, attr_long = 0;
+    allow_smem(join_walk_batch_kernel, &attr_walk);
+    allow_smem(join_long_kernel<true>, &attr_long);
+    join_walk_batch_kernel<<<b.nt, kJoinThreads, b.join_smem, s>>>(b);
+    if (b.n_heads && b.long_texts) {
+        const uint32_t blocks = b.n_heads * (b.recognize ? 1 : 2);
+        launch_dependent(join_long_kernel<false>, blocks, kFixThreads, 0, s, b);
+        launch_dependent(join_long_kernel<true>, blocks, kFixThreads, b.join_smem, s, b);
+    }
 }
 
 bool launch_join_walk(const Params &p, cudaStream_t s, int sm_count) {

@@ -144,8 +144,12 @@ struct WalkBatch {
     uint32_t recognize;
     size_t heads_smem, walk_smem, join_smem, gather_smem;
     const Params *texts;            // every text of the batch (those of other groups have rvar 0)
+    uint32_t *general;              // set when a long text has chunks whose runs never met; zeroed with the queues
     uint32_t nt;
+    uint32_t long_texts;            // some text has more than kJoinChunks chunks
 };
+// Chunks of a text up to which one block evaluates those whose runs never met.
+constexpr uint32_t kJoinChunks = 2048;
 enum Queue { Q_REACH = 0, Q_MERGE = 1, kQueues = 4 };
 
 // The text owning flat unit j: the last text whose first unit is <= j.

@@ -77,3 +77,27 @@ def test_batch(lib, name, chunk_len):
             exact = table[ids]
             assert int(st.item()) == (0 if serial.accepted(exact) else 1), (j, h.size)
             assert np.array_equal(rx.decode(outs[j].cpu().numpy(), kinds[j]), exact), (j, h.size)
+
+
+@pytest.mark.parametrize("recognize", [False, True])
+@pytest.mark.parametrize("more", [0, 1])
+def test_groups_beside_a_lane_walk(lib, more, recognize):
+    """Groups of small tables beside one that takes the lane walk, each of 1 MiB
+    in all (they join it) or of a byte more (they do not), in texts of many sizes."""
+    Batch, Regex = lib
+    log = W.log_text(300_000, seed=5)
+    items = [("log", W.LOG_RE, log), ("log", W.LOG_RE, log[:1].copy())]
+    for name in ("aa", "six", "dna"):
+        pattern, make = CASES[name]
+        sizes = [7, 600, 8194, 66_000, 280_000]
+        sizes.append((1 << 20) + more - sum(sizes))
+        items += [(name, pattern, make(n, n)) for n in sizes]
+    rxs = {name: Regex(pattern) for name, pattern, _ in items}
+    texts = [torch.from_numpy(h).cuda() for _, _, h in items]
+    b = Batch([rxs[name] for name, _, _ in items], [h.size for _, _, h in items], recognize_only=recognize)
+    outs, status, _ = b.parse(texts)
+    torch.cuda.synchronize()
+    for j, (name, _, h) in enumerate(items):
+        cols, st, _ = rxs[name].parse(texts[j], chunk_len=256, reach_shape=2)
+        assert int(status[j].item()) == int(st.item()), (name, h.size)
+        assert recognize or torch.equal(outs[j], cols), (name, h.size)
