@@ -919,7 +919,7 @@ struct re_batch {
     struct Group {
         re_handle *h = nullptr;
         uint32_t tmode = 0, ms = 0, enc_in_smem = 0, cb = 1;
-        bool walk = false;              // the lane walk (with per-position states unless recognizing)
+        bool can_walk = false, walk = false;   // the lane walk (with per-position states unless recognizing)
         uint32_t per = 0, logr = 0;     // heads round, table copies of the walk
         re_slpf_kind kind = RE_SLPF_DENSE;
         std::vector<uint32_t> members;  // caller indices, longest chunks first
@@ -990,6 +990,8 @@ Params group_like(const re_batch::Group &g, bool recognize) {
     q.mat = g.walk && !recognize ? 1u : 0u;
     return q;
 }
+
+constexpr uint64_t kShareWalk = 1 << 20;       // bytes of a group that joins the lane walk of others
 
 // Blocks for each weight, about `budget` in all and at least one each, at most
 // cap[j]: by share, then the rest to whoever has the most per block.
@@ -1159,7 +1161,8 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
             // encoder fits shared memory.  Where runs can stay apart, one 64 MiB text of a batch took
             // 38 ms by the lane walk and 0.34 by warp pairs (genome RE; recognized 40.6 and 0.125),
             // 16 of 4 MiB 2.85 and 0.36; 16 texts of 4 MiB under (aa)* 7.8 and 5.9.
-            g.walk = walk_first(h) && (b->recognize || mat_gather_smem(group_like(g, false)) <= kSmemMergeMax);
+            g.can_walk = walks(h) && (b->recognize || mat_gather_smem(group_like(g, false)) <= kSmemMergeMax);
+            g.walk = g.can_walk && walk_first(h);
             b->groups.push_back(std::move(g));
             gbytes.push_back(0);
         }
@@ -1168,8 +1171,16 @@ re_status re_batch_plan(re_handle *const *hs, const uint64_t *lens, uint32_t cou
         b->groups[it->second].members.push_back(j);
         gbytes[it->second] += lens[j];
     }
+    // Small groups share the launches of a lane walk that other groups need anyway: two of the 16
+    // REs of a served batch by launches of their own, 288 us instead of 245.
+    bool any = false;
+    for (const auto &g : b->groups) any = any || g.walk;
     uint64_t walk_bytes = 0;                                 // the lane-walk groups run at once
-    for (size_t j = 0; j < b->groups.size(); ++j) walk_bytes += b->groups[j].walk ? gbytes[j] : 0;
+    for (size_t j = 0; j < b->groups.size(); ++j) {
+        re_batch::Group &g = b->groups[j];
+        g.walk = g.walk || (any && g.can_walk && gbytes[j] <= kShareWalk);
+        walk_bytes += g.walk ? gbytes[j] : 0;
+    }
     // chunk lengths, then members longest chunks first
     for (uint32_t j = 0; j < count; ++j) {
         re_batch::Text &t = b->texts[j];
