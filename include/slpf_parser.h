@@ -348,7 +348,11 @@ re_status re_parse_static(re_handle *h, const uint8_t *d_text, uint64_t len, re_
  * group inside an ambiguous iteration (an ORF whose codon star also matches
  * stop codons) can have a number of matches, and a cost, quadratic in the
  * text length.
- * d_workspace: re_match_workspace_size bytes, 256-byte aligned.            */
+ * d_workspace, 256-byte aligned: re_match_workspace_size bytes, about half a
+ * byte per text byte, most of it for the spans that the counting pass finds.
+ * Less is taken too, down to the counts alone (8 bytes per 2048 columns and
+ * 8 per 2^21, each rounded up to 256): the columns are then visited again
+ * for the pairs.                                                            */
 re_status re_match_workspace_size(const re_handle *h, uint64_t len, uint64_t *bytes);
 re_status re_matches(re_handle *h, const re_slpf *slpf, uint64_t len, uint32_t group, uint64_t *d_pairs,
                      uint64_t cap_pairs, uint64_t *d_count, void *d_workspace, uint64_t workspace_bytes,

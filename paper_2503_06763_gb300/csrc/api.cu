@@ -787,7 +787,7 @@ extern "C" re_status re_parse_host(re_handle *h, const uint8_t *text, uint64_t l
 // ------------------------------------------------------------------ match extraction
 extern "C" re_status re_match_workspace_size(const re_handle *h, uint64_t len, uint64_t *bytes) {
     if (!h || !bytes) { set_error("null argument"); return RE_E_INVALID_ARG; }
-    *bytes = match_workspace_bytes(len);
+    *bytes = match_workspace_bytes(len, true);
     return RE_OK;
 }
 
@@ -826,7 +826,7 @@ extern "C" re_status re_matches(re_handle *h, const re_slpf *slpf, uint64_t len,
             if (kp[x] == 1 && std::find(kp.begin() + x + 1, kp.end(), -1) != kp.end()) { a.whole[w] |= bit; break; }
     }
     if (!group || !is_group) { set_error("no group with this number (an operator node of the numbered RE)"); return RE_E_INVALID_ARG; }
-    if (!d_workspace || workspace_bytes < match_workspace_bytes(len) || ((uintptr_t)d_workspace & 255)) {
+    if (!d_workspace || workspace_bytes < match_workspace_bytes(len, false) || ((uintptr_t)d_workspace & 255)) {
         set_error("workspace missing, too small or not 256-byte aligned");
         return RE_E_CAPACITY;
     }
@@ -848,7 +848,7 @@ extern "C" re_status re_matches(re_handle *h, const re_slpf *slpf, uint64_t len,
     a.pairs = d_pairs;
     a.cap = cap_pairs;
     a.count = d_count;
-    launch_matches(a, d_workspace, (cudaStream_t)stream, sm_count_of(h->device));
+    launch_matches(a, d_workspace, workspace_bytes, (cudaStream_t)stream, sm_count_of(h->device));
     CUDA_TRY(cudaGetLastError(), "match launch");
     return RE_OK;
 }

@@ -532,16 +532,15 @@ struct MatchArgs {
     const int32_t *status;                    // parse status: anything but RE_OK gives no matches
     uint64_t *cnt;                            // [G] pairs per tile, then their exclusive offsets
     uint64_t *bsum;                           // [ceil(G / kScanBlock)] block totals, then offsets
-    uint64_t *total;                          // [1] all matches
-    uint32_t *recs;                           // [G][kRecs] the count pass's spans of each tile
+    uint32_t *recs;                           // [G][kRecs] the count pass's spans of each tile, or null
     uint64_t G;
     uint64_t *pairs;                          // [cap][2]
     uint64_t cap;
-    uint64_t *count;
+    uint64_t *count;                          // [1] all matches
 };
 
-size_t match_workspace_bytes(uint64_t n);
-void launch_matches(MatchArgs a, void *ws, cudaStream_t s, int sm_count);
+size_t match_workspace_bytes(uint64_t n, bool records);
+void launch_matches(MatchArgs a, void *ws, size_t ws_bytes, cudaStream_t s, int sm_count);
 
 // Batch launchers: one launch per phase for every text of the group.
 void launch_batch_init(const Params *texts, uint32_t nt, uint32_t *queues, uint32_t nq, cudaStream_t s);

@@ -258,16 +258,15 @@ __global__ void __launch_bounds__(kMatchThreads) match_kernel(const __grid_const
     const bool vec = (reinterpret_cast<uintptr_t>(a.cols) & 15) == 0;
     const uint64_t warps = (uint64_t)gridDim.x * (kMatchThreads / 32);
     for (uint64_t g = (uint64_t)blockIdx.x * (kMatchThreads / 32) + warp; g < a.G; g += warps) {
-        uint32_t *recs = a.recs + g * kRecs;
+        uint32_t *recs = a.recs ? a.recs + g * kRecs : nullptr;
         uint64_t off = 0;                                     // the tile's matches so far
-        bool fit = true;                                      // ... are all in its records
+        bool fit = recs != nullptr;                           // ... are all in its records
         const uint64_t first = WRITE ? a.cnt[g] + a.bsum[g / kScanBlock] : 0;   // matches before the tile
         if (WRITE) {
-            const uint64_t after = g + 1 == a.G ? a.total[0] : a.cnt[g + 1] + a.bsum[(g + 1) / kScanBlock];
+            const uint64_t after = g + 1 == a.G ? a.count[0] : a.cnt[g + 1] + a.bsum[(g + 1) / kScanBlock];
             off = after - first;
-            if (g + 1 == a.G && lane == 0) *a.count = after;
             if (off == 0 || first >= a.cap) continue;
-            if (off <= kRecs && recs[0] != kNoRecs) {
+            if (recs && off <= kRecs && recs[0] != kNoRecs) {
                 const uint32_t m = (uint32_t)min(off, a.cap - first);
                 for (uint32_t q = lane; q < m; q += 32) {
                     const uint32_t r = recs[q];
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(kMatchThreads) match_kernel(const __grid_const
         }
         if (!WRITE && lane == 0) {
             a.cnt[g] = off;
-            if (!fit) recs[0] = kNoRecs;
+            if (recs && !fit) recs[0] = kNoRecs;
         }
     }
 }
@@ -394,23 +393,26 @@ __global__ void scan_totals_kernel(uint64_t *v, uint64_t n, uint64_t *total) {
 }  // namespace
 
 namespace {
-// Workspace: per-tile counts, block sums of the scan, the total, the records.
+// Workspace: per-tile counts, block sums of the scan, the records.  Without room
+// for the records the write pass visits every tile again.
 struct MatchWorkspace {
     uint64_t G, nb;
-    size_t bsum, total, recs, bytes;
+    size_t bsum, recs, bytes;
     explicit MatchWorkspace(uint64_t n) {
         auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
         G = n / kTile + 1;                                    // tiles of kTile start columns, a warp each
         nb = (G + kScanBlock - 1) / kScanBlock;
         bsum = up(G * 8);
-        total = bsum + up(nb * 8);
-        recs = total + 256;
+        recs = bsum + up(nb * 8);
         bytes = recs + up(G * kRecs * 4);
     }
 };
 }  // namespace
 
-size_t match_workspace_bytes(uint64_t n) { return MatchWorkspace(n).bytes; }
+size_t match_workspace_bytes(uint64_t n, bool records) {
+    const MatchWorkspace w(n);
+    return records ? w.bytes : w.recs;
+}
 
 template <int W, int CB>
 static void run_matches(const MatchArgs &a, uint64_t nb, cudaStream_t s, int sm_count) {
@@ -426,7 +428,7 @@ static void run_matches(const MatchArgs &a, uint64_t nb, cudaStream_t s, int sm_
     const uint64_t gw = std::min<uint64_t>(want, (uint64_t)std::max(pw, 1) * sm_count);
     match_kernel<W, CB, false><<<(uint32_t)gc, kMatchThreads, smem, s>>>(a);
     scan_block_kernel<<<(uint32_t)nb, kScanBlock, 0, s>>>(a.cnt, a.G, a.bsum);
-    scan_totals_kernel<<<1, kScanBlock, 0, s>>>(a.bsum, nb, a.total);
+    scan_totals_kernel<<<1, kScanBlock, 0, s>>>(a.bsum, nb, a.count);
     match_kernel<W, CB, true><<<(uint32_t)gw, kMatchThreads, smem, s>>>(a);
 }
 
@@ -444,15 +446,14 @@ static void matches_of_width(const MatchArgs &a, uint64_t nb, cudaStream_t s, in
 // write pass 27 us, where a lane per column in both passes took 0.79 and 1.42
 // ms.  The count pass is bound by instruction issue (74 % of the slots; 740
 // instructions per warp and 512 columns), the write pass by its 50 MB of pairs.
-void launch_matches(MatchArgs a, void *ws, cudaStream_t s, int sm_count) {
+void launch_matches(MatchArgs a, void *ws, size_t ws_bytes, cudaStream_t s, int sm_count) {
     const MatchWorkspace w(a.n);
     uint8_t *p = static_cast<uint8_t *>(ws);
     const uint64_t nb = w.nb;
     a.G = w.G;
     a.cnt = reinterpret_cast<uint64_t *>(p);
     a.bsum = reinterpret_cast<uint64_t *>(p + w.bsum);
-    a.total = reinterpret_cast<uint64_t *>(p + w.total);
-    a.recs = reinterpret_cast<uint32_t *>(p + w.recs);
+    a.recs = ws_bytes >= w.bytes ? reinterpret_cast<uint32_t *>(p + w.recs) : nullptr;
     if (a.W <= 1) matches_of_width<1>(a, nb, s, sm_count);
     else if (a.W <= 2) matches_of_width<2>(a, nb, s, sm_count);
     else if (a.W <= 4) matches_of_width<4>(a, nb, s, sm_count);
