@@ -32,6 +32,7 @@ constexpr uint32_t kHeadWindow = 144;       // bytes of a chunk staged, from its
 constexpr uint32_t kHeadStride = 148;       // their stride: an odd number of words, so lanes hit different banks
 constexpr int kRuns = 4;
 constexpr uint32_t kWideBytes = 32;         // bytes a warp walks a chunk's slots
+constexpr uint32_t kWideRuns = 8;           // runs a lane takes on from there
 
 // Drop dead runs and merge runs in equal states (their slot sets are joined);
 // unused runs hold the empty state.
@@ -74,7 +75,8 @@ struct GroupTexts {
 struct HeadShared {
     uint32_t ti[kHeadChunks];                // the text of each chunk of the round
     uint8_t text[kHeadChunks * kHeadStride];
-    uint32_t s[kRuns][kHeadChunks], k[kRuns][kHeadChunks], cnt[kHeadChunks], col[kHeadChunks];
+    uint32_t s[kRuns][kHeadChunks], k[kWideRuns][kHeadChunks], cnt[kHeadChunks], col[kHeadChunks];
+    uint8_t s8[kWideRuns][kHeadChunks];      // states of a chunk with more than kRuns runs, their slot sets in k
     uint16_t wide[kHeadChunks];              // chunks of this round with more than kRuns slots: slots << 8 | chunk
     uint32_t pr[kHeadChunks], nwide;
 };
@@ -104,49 +106,103 @@ __device__ __forceinline__ void head_word(const LaneTab &T, uint32_t w, uint32_t
     for (int q = 0; q < 4; ++q) head_byte<W>(T, __byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)), s);
 }
 
-// The end states of a chunk's slots, eight at a time from its edge, by one lane:
-// where more runs than a lane keeps are apart after kWideBytes.  They hardly
-// ever meet later, so they are not compared; a state is a byte, and the eight are
-// kept in two words.  A warp per chunk walking them on to its end, most of its
-// lanes idle, made the heads of 64 MiB of a's under twenty (c{6}) 3.4 ms; now 0.45.
+// Eight runs of a lane over columns [c, to) (right to left where not FWD): a state
+// is a byte, and the eight are kept in two words.
+template <bool FWD>
+__device__ __forceinline__ void walk_eight(const LaneTab &T, const uint8_t *x, uint32_t len, uint32_t &c, uint32_t to,
+                                           uint32_t (&s)[2]) {
+    auto step = [&](uint32_t byte) {
+        const uint32_t col = lane_col<0>(T, byte);
+        uint32_t v[8];
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u) v[u] = lds8(__byte_perm(s[u >> 2], 0u, 0x4440u | (u & 3)) * T.rowb + col);
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h)
+            s[h] = __byte_perm(__byte_perm(v[4 * h], v[4 * h + 1], 0x0040u), __byte_perm(v[4 * h + 2], v[4 * h + 3], 0x0040u), 0x5410u);
+    };
+#pragma unroll 1
+    while (c != to && (s[0] | s[1])) {
+        const uint32_t left = FWD ? to - c : c - to;
+        if ((c & 3) == 0 && left >= 4) {
+            const uint32_t a4 = FWD ? c : c - 4;
+            if ((c & 127) == 0 && (FWD ? len - c : c) > 256) prefetch_l2(x + (FWD ? c + 128 : c - 256));
+            const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(x + a4));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) step(__byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)));
+            c = FWD ? c + 4 : c - 4;
+        } else {
+            step(__ldg(x + (FWD ? c : c - 1)));
+            c = FWD ? c + 1 : c - 1;
+        }
+    }
+    c = to;                                                   // no run was left
+}
+__device__ __forceinline__ uint32_t state_of(const uint32_t (&s)[2], uint32_t u) { return (s[u >> 2] >> (8 * (u & 3))) & 0xFFu; }
+
+// A chunk with more than kRuns and at most kWideRuns runs after kWideBytes: a lane
+// goes on with them, equal ones joined after every unit, until kRuns are left
+// (returned in S) or the chunk ends (every slot's end state written).  A warp per
+// chunk going on to that point, most of its lanes idle, made the heads of 64 MiB of
+// a's under twenty (c{6}) 3.4 ms (0.45 now); the genome RE, whose runs meet after some
+// 450 bytes, has 5 to 8 of them for a while (256 MiB by the lane walk 778 us, and 1554
+// with every such chunk walked to its end).
+template <bool FWD>
+__device__ void eight_runs(const LaneTab &T, HeadShared &S, const uint8_t *x, uint32_t len, uint32_t q, uint32_t ms, uint32_t *R) {
+    uint32_t s[2], c = S.col[q], n = kWideRuns;
+#pragma unroll
+    for (uint32_t u = 0; u < 8; ++u) s[u >> 2] = (u & 3 ? s[u >> 2] : 0u) | (uint32_t)S.s8[u][q] << (8 * (u & 3));
+    while ((FWD ? c < len : c > 0) && n > (uint32_t)kRuns) {
+        walk_eight<FWD>(T, x, len, c, FWD ? min((c / kUnit + 1) * kUnit, len) : (c - 1) / kUnit * kUnit, s);
+        n = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u) {
+            const uint32_t v = state_of(s, u);
+            bool own = v != 0;
+#pragma unroll
+            for (uint32_t e = 0; e < u; ++e)
+                if (v && state_of(s, e) == v) {
+                    S.k[e][q] |= S.k[u][q];
+                    s[u >> 2] &= ~(0xFFu << (8 * (u & 3)));
+                    own = false;
+                    break;
+                }
+            n += own;
+        }
+    }
+    S.col[q] = c;
+    S.cnt[q] = min(n, (uint32_t)kRuns + 1);
+    uint32_t at = 0;
+    if (n <= (uint32_t)kRuns) {
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u)
+            if (state_of(s, u)) { S.s[at][q] = state_of(s, u); S.k[at][q] = S.k[u][q]; ++at; }
+        for (; at < (uint32_t)kRuns; ++at) S.s[at][q] = S.k[at][q] = 0;
+    } else {
+        for (uint32_t j = 0; j < ms; ++j) {
+            uint32_t v = 0;
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u)
+                if (state_of(s, u) && (S.k[u][q] >> j & 1u)) v = state_of(s, u);
+            R[j] = v;
+        }
+    }
+}
+
+// The end states of a chunk's slots, eight at a time from its edge, by a lane: where
+// even more runs are apart after kWideBytes.
 template <bool FWD>
 __device__ void slots_to_end(const LaneTab &T, const uint8_t *x, uint32_t len, const uint32_t *starts, uint32_t m,
                              uint32_t ms, uint32_t *R) {
 #pragma unroll 1
     for (uint32_t j = 0; j < ms; j += 8) {
-        uint32_t s[2] = {0, 0};
+        uint32_t s[2] = {0, 0}, c = FWD ? 1u : len - 1;
 #pragma unroll
         for (uint32_t u = 0; u < 8; ++u)
             if (j + u < m) s[u >> 2] |= __ldg(starts + j + u) << (8 * (u & 3));
-        auto step = [&](uint32_t byte) {
-            const uint32_t col = lane_col<0>(T, byte);
-            uint32_t v[8];
-#pragma unroll
-            for (uint32_t u = 0; u < 8; ++u) v[u] = lds8(__byte_perm(s[u >> 2], 0u, 0x4440u | (u & 3)) * T.rowb + col);
-#pragma unroll
-            for (uint32_t h = 0; h < 2; ++h)
-                s[h] = __byte_perm(__byte_perm(v[4 * h], v[4 * h + 1], 0x0040u), __byte_perm(v[4 * h + 2], v[4 * h + 3], 0x0040u), 0x5410u);
-        };
-        uint32_t c = FWD ? 1u : len - 1;
-        const uint32_t end = FWD ? len : 0u;
-#pragma unroll 1
-        while (c != end && (s[0] | s[1])) {
-            const uint32_t left = FWD ? end - c : c;
-            if ((c & 3) == 0 && left >= 4) {
-                const uint32_t a4 = FWD ? c : c - 4;
-                if ((a4 & 127) == (FWD ? 0u : 124u) && left > 128) prefetch_l2(x + (FWD ? c + 128 : c - 132));
-                const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(x + a4));
-#pragma unroll
-                for (int q = 0; q < 4; ++q) step(__byte_perm(w, 0u, 0x4440u | (uint32_t)(FWD ? q : 3 - q)));
-                c = FWD ? c + 4 : c - 4;
-            } else {
-                step(__ldg(x + (FWD ? c : c - 1)));
-                c = FWD ? c + 1 : c - 1;
-            }
-        }
+        walk_eight<FWD>(T, x, len, c, FWD ? len : 0u, s);
 #pragma unroll
         for (uint32_t u = 0; u < 8; ++u)
-            if (j + u < ms) R[j + u] = (s[u >> 2] >> (8 * (u & 3))) & 0xFFu;
+            if (j + u < ms) R[j + u] = state_of(s, u);
     }
 }
 
@@ -229,8 +285,13 @@ __device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint
                 if (lane == 0) { S.cnt[q] = kRuns + 1; S.col[q] = c; }
                 break;
             }
-            if ((FWD ? c : ch.len - c) >= kWideBytes) {       // a lane takes the slots, from the edge
-                if (lane == 0) { S.cnt[q] = kRuns + 2; S.col[q] = c; }
+            if ((FWD ? c : ch.len - c) >= kWideBytes) {       // a lane takes the runs, or all slots from the edge
+                if (n <= kWideRuns) {
+                    const uint32_t at = __popc(lead & ((1u << lane) - 1));
+                    if (is_lead) { S.s8[at][q] = (uint8_t)v; S.k[at][q] = same; }
+                    if (lane >= n && lane < kWideRuns) { S.s8[lane][q] = 0; S.k[lane][q] = 0; }
+                }
+                if (lane == 0) { S.cnt[q] = n <= kWideRuns ? kRuns + 3 : kRuns + 2; S.col[q] = c; }
                 break;
             }
         }
@@ -253,11 +314,18 @@ __device__ void head_round(const Src &src, const LaneTab &T, HeadShared &S, uint
         } else if (valid) {
             n = S.cnt[q];
             c = S.col[q];
+            if (n > (uint32_t)kRuns + 1) {
+                uint32_t *R = (FWD ? p.w.Rf : p.w.Rb) + (size_t)ch.i * ms;
+                if (n == kRuns + 3) {
+                    eight_runs<FWD>(T, S, p.x + ch.base, ch.len, q, ms, R);
+                    n = S.cnt[q];
+                    c = S.col[q];
+                } else {
+                    slots_to_end<FWD>(T, p.x + ch.base, ch.len, starts + (size_t)S.pr[q] * ms,
+                                      __ldg((FWD ? t.fSlotCount : t.bSlotCount) + S.pr[q]), ms, R);
+                }
+            }
             all = n > (uint32_t)kRuns;
-            if (n == kRuns + 2)
-                slots_to_end<FWD>(T, p.x + ch.base, ch.len, starts + (size_t)S.pr[q] * ms,
-                                  __ldg((FWD ? t.fSlotCount : t.bSlotCount) + S.pr[q]), ms,
-                                  (FWD ? p.w.Rf : p.w.Rb) + (size_t)ch.i * ms);
             open = !all && (FWD ? c < ch.len : c > 0);
 #pragma unroll
             for (int j = 0; j < kRuns; ++j)
@@ -348,7 +416,7 @@ __global__ void __launch_bounds__(kHeadThreads) heads_kernel(const __grid_consta
 }
 
 // Every lane-walk group of a batch: a block takes rounds of one group's chunks.
-__global__ void __launch_bounds__(kHeadThreads) heads_batch_kernel(const __grid_constant__ WalkBatch b) {
+__global__ void __launch_bounds__(kHeadThreads, 8) heads_batch_kernel(const __grid_constant__ WalkBatch b) {
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ __align__(128) uint8_t cls[256];
     __shared__ HeadShared S;

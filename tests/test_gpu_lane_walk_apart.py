@@ -5,6 +5,7 @@ Against the oracle."""
 import numpy as np
 import pytest
 
+import workloads as W
 from oracle import serial
 from oracle.re_front import compile_re
 
@@ -68,3 +69,24 @@ def test_slices(lib, name, n):
             assert accepted == serial.accepted(want)
             assert (stats.cpu().numpy() == (0 if accepted else 1)).all()
             assert np.array_equal(rx.decode(cols.cpu().numpy(), rx.layout(1)[0]), want), parts
+
+
+@pytest.mark.parametrize("k", [256, 576, 1024, 4096])
+@pytest.mark.parametrize("n", [4095, 70_001, 200_003])
+def test_runs_that_meet_late(lib, n, k):
+    """The genome RE has up to eight runs for some hundred bytes: they meet in a
+    lane's share of the chunk, down to few enough for the rest or to its end."""
+    Regex, _ = lib
+    rx, c = Regex(W.DNA_RE), compile_re(W.DNA_RE)
+    host = W.dna_text(n, seed=n + k, mean_gap=700)
+    for spoil in (None, n - 60):
+        if spoil is not None:
+            host[spoil] = ord("N")
+        ids, table = serial.parse_ids(c, host)
+        want = table[ids]
+        t = torch.from_numpy(host).cuda()
+        cols, st, kind = rx.parse(t, chunk_len=k, reach_shape=1)
+        _, rst, _ = rx.parse(t, chunk_len=k, reach_shape=1, recognize_only=True)
+        torch.cuda.synchronize()
+        assert int(st.item()) == int(rst.item()) == (0 if serial.accepted(want) else 1)
+        assert np.array_equal(rx.decode(cols.cpu().numpy(), kind), want)
