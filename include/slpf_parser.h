@@ -47,7 +47,8 @@ typedef enum {
     RE_E_INFINITE_AMBIGUITY = -3,  /* an iterated sub-RE derives the empty text (Sect. 2.1, App. A)
                                       and re_compile_opts.sample_limit is 0 */
     RE_E_TOO_MANY_STATES = -4,     /* automaton exceeds re_compile_opts.max_states */
-    RE_E_NOMEM = -5,               /* host or device allocation failed (re_compile only) */
+    RE_E_NOMEM = -5,               /* host or device allocation failed (re_compile, re_batch_plan, re_server_create,
+                                      re_slpf_dfa_encode) */
     RE_E_CUDA = -6,                /* CUDA runtime error; see re_last_error() */
     RE_E_TIMEOUT = -7,             /* status word only: a bounded device wait ran out (the join's grid barrier) */
     RE_E_CAPACITY = -8,            /* an output / workspace buffer is smaller than required */
@@ -202,7 +203,8 @@ typedef struct {
     uint32_t inf_ambiguous;   /* 1 when the RE is infinitely ambiguous (its SLPFs are samples) */
     uint32_t sample_limit;    /* the compile option's sample_limit */
     uint32_t ascii_rows;      /* 1 when every byte class holding a byte >= 128 also holds one
-                                 below 128 (automata of at most 256 states per direction) */
+                                 below 128 (automata of at most 256 states per direction);
+                                 for information, nothing is chosen by it */
     uint32_t reach_shapes;    /* bit v set: reach shape v (RE_PARSE_REACH) runs for this automaton */
 } re_info;
 
@@ -246,22 +248,24 @@ re_status re_parse(re_handle *h, const uint8_t *d_text, uint64_t len, re_stream 
                    const re_parse_opts *opts);
 
 /* ---------------------------------------------------------------- batches
- * Many texts, each under its own compiled RE, parsed together: the texts
- * that share a handle form a group, and every phase of a group is one kernel
- * launch over all its texts (reach tiles of 32 chunks, chunks, and merge
- * tiles of 32 column groups, handed out by device work counters), instead of
- * one launch per phase and text.  Results are those of re_parse on each text
- * (Sect. 3.2); the chunk length of each text is chosen from its length and
- * its group's total length (re_batch_chunk_len reports it).
+ * Many texts, each under its own compiled RE, parsed together, with one kernel
+ * launch per phase instead of one per phase and text: the texts that share a
+ * handle form a group; the groups for which a single text would take the lane
+ * walk share its launches (and beside them other groups of automata of at most
+ * 256 states whose texts are at most 1 MiB in all), every other group has
+ * launches of its own (reach tiles of 32 chunks, chunks, and merge tiles of 32
+ * column groups, handed out by device work counters).  Results are those of
+ * re_parse on each text (Sect. 3.2); the chunk length of each text is chosen
+ * from its length and its group's total length (re_batch_chunk_len reports it).
  *
  * Use: re_batch_plan (host only; sizes, chunk lengths, a pinned descriptor
  * buffer) -> re_batch_workspace_size -> re_parse_batch (binds text, output
  * and workspace pointers, encodes each text's tensor maps, uploads the
  * descriptors, enqueues the kernels) -> re_batch_run to parse the same bound
  * buffers again (kernels only, nothing copied) -> re_batch_free.
- * A batch of 64 MiB or more under several REs runs its groups on up to four
- * streams of its own, forked from and joined back into the caller's stream
- * by events (a CUDA graph capture of the call captures them too).           */
+ * Several groups with launches of their own, of 64 MiB or more in all, run on
+ * up to four streams of the plan's, forked from and joined back into the
+ * caller's stream by events (a CUDA graph capture of the call captures them too). */
 typedef struct re_batch re_batch;       /* opaque: a planned batch */
 
 /* Plan count texts: text j has lens[j] bytes and is parsed under hs[j] (all

@@ -57,11 +57,11 @@ uint32_t table_mode(const DevTables &t);
 // The lane walk (RE_PARSE_REACH shape 1) is the built-in choice for automata of
 // at most 256 states: where their two-byte tables do not fit shared memory, and
 // where they do if every text makes a chunk's runs meet within kMeetMax letters
-// ((a|b|ab)* at 1 MiB 36 us against 59 for warp pairs, at 256 MiB 432 against
-// 470).  With small tables and runs that can stay apart, warp pairs are the
-// better ones: they take two bytes a lookup and the walk's join evaluates the
-// chunks whose runs never met ((aa)* at 64 MiB 475 us against 612 for the lane
-// walk, the genome RE at 256 MiB 594 against 791).
+// ((a|b|ab)* on the device: 1 MiB 34 us against 40 for warp pairs, 256 MiB 415
+// against 460).  With small tables and runs that can stay apart, warp pairs are
+// the better ones: they take two bytes a lookup and record the runs until they
+// meet, where the lane walk goes through such chunks once more ((aa)* at 64 MiB
+// 486 us against 593 for the lane walk, the genome RE at 256 MiB 568 against 778).
 constexpr uint32_t kMeetMax = 64;
 bool walk_first(const re_handle *h) {
     return walks(h) && (table_mode(h->dev) == TM_SMEM || h->host.meet <= kMeetMax);
@@ -87,10 +87,11 @@ uint32_t plain_chunk(uint64_t n, int sms) { return chunk_for(n, (uint64_t)sms * 
 // Warp pairs: the chunks of plain_chunk, or fewer where half of them or less
 // are better: a chunk's bytes are walked one after another, 24 ns each, and
 // each chunk costs the join about 4 ns when byte states make it a scan over all
-// chunks, and under 2 ns when it is not; the sum is least at k = sqrt(n / 8)
-// and about sqrt(n / 16).  Genome RE, 16 MiB: 320-byte chunks 254 us, 1472 159;
-// 1 MiB: 256 130, 384 120; 256 MiB: 5824 616, 4608 592.  (a|b)*a(a|b)^9, 16
-// MiB: 320 178, 1024 128.
+// chunks (less by units of several), and under 2 ns when it is not; the sum is
+// least at k = sqrt(n / 8) and about sqrt(n / 16).  Genome RE, 16 MiB: 320-byte
+// chunks 346 us, 1472 152; 1 MiB: 256 133, 384 118; 64 MiB: 1152 310, 2944 258;
+// 256 MiB: 5824 593, 4608 580.  (aa)*, 64 MiB: 1152 502, 2944 494.
+// (a|b)*a(a|b)^9, 16 MiB: 320 178, 1024 128.
 uint32_t choose_chunk(const re_handle *h, uint64_t n, int sms, const re_parse_opts *opts) {
     if (opts && opts->chunk_len) return opts->chunk_len;
     const bool rec = opts && (opts->flags & RE_PARSE_RECOGNIZE_ONLY);
@@ -490,13 +491,7 @@ re_status workspace_rule_bytes(const re_handle *h, uint64_t len, const re_parse_
     *bytes = layout_for(h, len, k, mat_for(h, opts)).total;
     return RE_OK;
 }
-}  // namespace slpf
 
-extern "C" {
-
-}  // extern "C"
-
-namespace slpf {
 // A slice of a sharded text: its entry states (forward at its start,
 // backward at its end; I and F for a whole text), and in map mode the
 // device buffer of its maps and its SHARD_* flags.

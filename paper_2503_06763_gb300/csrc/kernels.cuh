@@ -74,7 +74,8 @@ struct Params {
                                     // chains, one thread each
     uint32_t scan_stall;            // test hook: one block of the scan never reaches its first barrier
     uint32_t mat;                   // reach writes every position's state once its runs have met; the
-                                    // fix-up fills the positions before; build & merge is a gather
+                                    // positions before are filled by the fix-up, or by the walk of the
+                                    // chunk before (the lane walk); build & merge is a gather
     uint32_t state_tma;             // reach stores its state rows through TMA (mat)
     uint32_t rvar;                  // reach shape (RE_PARSE_REACH): 1 the lane walk; 2 / 3 warp pairs, 3 / 2 stages; 4 one lane per chunk
     uint32_t rstages;               // TMA ring stages of the warp-pair and one-lane shapes
@@ -95,7 +96,8 @@ struct Params {
 };
 
 // TMA maps of the per-position state arrays FS and BS (mat): rows of k
-// positions (one chunk), boxes of 32 rows x 64 positions, SWIZZLE_64B.
+// positions (one chunk), boxes of 32 rows x 64 positions, SWIZZLE_64B (the lane
+// walk: 32 positions, SWIZZLE_32B).
 struct StateMaps {
     CUtensorMap f, b;
 };
@@ -496,8 +498,8 @@ __host__ __device__ inline size_t dict_bytes(const DevTables &t, uint32_t cb) {
 }
 bool launch_reach(const Params &p, const CUtensorMap &text_map, const StateMaps &smaps, cudaStream_t s, uint32_t ms,
                   int sm_count);
-// The lane walk over the groups of a batch: one launch per phase.  The *_plan
-// functions give what a group needs of each.
+// The lane walk over the groups of a batch: one launch per phase, and what a
+// group needs of each.
 void launch_heads_batch(const WalkBatch &b, cudaStream_t s);
 void launch_walk_batch(const WalkBatch &b, cudaStream_t s);
 void launch_join_walk_batch(const WalkBatch &b, cudaStream_t s);

@@ -13,12 +13,13 @@
 // no tiles and no barriers, but costs a wavefront per lane and access, 0.27 ms
 // at 256 MiB of log text.
 //
-// Measured (heads and walk together, log text): 11 MiB 47 us, 256 MiB 0.27 ms,
-// 1 GiB 0.97 ms = 4.3 TB/s of text read and states written, where one kernel
-// of byte-indexed tables that held a chunk's runs in registers and local
-// memory took 140 us, 0.37 ms and 1.10 ms and left the chunk heads to another.
-// What bounds it: issue slots (72 % busy, 11 instructions per byte step) and
-// the shared-memory pipe (73 %) together.
+// Measured (heads and walk together, log text): 11 MiB 45 us, 256 MiB 0.27 ms,
+// 1 GiB 0.94 ms (autotuned chunk length) = 3.4 TB/s of text read once and states
+// written, where one kernel of byte-indexed tables that held a chunk's runs in
+// registers and local memory took 140 us, 0.37 ms and 1.10 ms and left the chunk
+// heads to another.  What bounds it: issue slots (69 % busy, 11 instructions per
+// byte step) and the shared-memory pipe (70 %) together (256 MiB, the rule's
+// chunk length).
 #include <algorithm>
 #include <type_traits>
 
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1)
 // length and come longest first; dealt round-robin instead, 768 texts of 1 KiB
 // to 4 MiB took 0.52 ms; from the queue, and with whole tiles, 0.39 ms).
 template <int LOGR, bool OUT>
-__device__ void walk_group(const WalkBatch &b, const WalkGroup &g, const WalkSpan &sp, bool backward, uint8_t *sm, uint8_t *cls) {
+__device__ void walk_group(const WalkBatch &b, const WalkGroup &g, bool backward, uint8_t *sm, uint8_t *cls) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t fixed = 1024 + lane_table_bytes<LOGR>(g.t);  // warps this group's tables leave room for
     const uint32_t wpb = min(blockDim.x / 32, (uint32_t)((b.walk_smem - fixed) / kWalkWarpSmem));
@@ -295,16 +296,19 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 1) walk_batch_kernel(const __
     const WalkSpan sp = b.walk[pairs ? blockIdx.x >> 1 : blockIdx.x];
     const WalkGroup &g = b.groups[sp.group];
     switch (g.logr) {
-        case 5: walk_group<5, OUT>(b, g, sp, backward, sm, cls); break;
-        case 4: walk_group<4, OUT>(b, g, sp, backward, sm, cls); break;
-        case 2: walk_group<2, OUT>(b, g, sp, backward, sm, cls); break;
-        default: walk_group<0, OUT>(b, g, sp, backward, sm, cls); break;
+        case 5: walk_group<5, OUT>(b, g, backward, sm, cls); break;
+        case 4: walk_group<4, OUT>(b, g, backward, sm, cls); break;
+        case 2: walk_group<2, OUT>(b, g, backward, sm, cls); break;
+        default: walk_group<0, OUT>(b, g, backward, sm, cls); break;
     }
 }
 
 // Table copies: as many of 32, 16 or 4 as leave room for kWalkMinWarps warps.
 // With few tiles per block the walk is one chain's latency, and copying the
-// table costs more than its conflicts: one copy.
+// table costs more than its conflicts: one copy (heads and walk of log text: 64 KiB
+// 30 us with one copy and 49 with 32, 1 MiB 30 and 55; above the line 4 MiB 35 and
+// 40, 11 MiB and more by 32).  Random REs whose 32 copies leave 16 to 24 warps, 64
+// MiB: 84 to 88 us with 32 copies, 90 with 16, 103 with 4.
 constexpr uint32_t kWalkMinWarps = 12;
 int walk_logr(const DevTables &t, uint64_t tiles, uint64_t blocks) {
     if (tiles <= 2 * blocks) return 0;

@@ -495,8 +495,9 @@ class Regex:
 
 class Batch:
     """A planned batch (re_batch_plan): texts j of lens[j] bytes, each under
-    regexes[j].  ``parse`` binds CUDA tensors and enqueues every phase as one
-    launch per RE; ``run`` re-enqueues the kernels over the same buffers."""
+    regexes[j].  ``parse`` binds CUDA tensors and enqueues the phases, each one
+    launch over the texts of all REs that take the lane walk and one per RE for
+    the others; ``run`` re-enqueues the kernels over the same buffers."""
 
     def __init__(self, regexes, lens, kind: str = "auto", chunk_len: int = 0, recognize_only: bool = False):
         self.regexes = list(regexes)
