@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kBlockThreads) join_walk_kernel(const __grid_c
 // The same for every text of a batch's lane-walk groups, a block per text, its
 // lower half forward and its upper half backward: chunks whose runs never met are
 // evaluated in chains.  Longer texts with such chunks are left to join_long_kernel.
-constexpr uint32_t kJoinThreads = 256;
+constexpr uint32_t kJoinThreads = 128;
 __global__ void __launch_bounds__(kJoinThreads) join_walk_batch_kernel(const __grid_constant__ WalkBatch b) {
     extern __shared__ __align__(16) uint8_t sm[];
     const Params &p = b.texts[blockIdx.x];

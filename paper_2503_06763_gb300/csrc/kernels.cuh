@@ -150,8 +150,10 @@ struct WalkBatch {
     uint32_t nt;
     uint32_t long_texts;            // some text has more than kJoinChunks chunks
 };
-// Chunks of a text up to which one block evaluates those whose runs never met.
-constexpr uint32_t kJoinChunks = 2048;
+// Chunks of a text up to which one block evaluates those whose runs never met:
+// a text of 1 MiB in the shortest chunks.  The launches for longer texts cost a
+// batch 2 to 3 us, 68.5 us instead of 66 for 64 texts of up to 1 MiB under one RE.
+constexpr uint32_t kJoinChunks = 4096;
 enum Queue { Q_REACH = 0, Q_MERGE = 1, kQueues = 4 };
 
 // The text owning flat unit j: the last text whose first unit is <= j.
